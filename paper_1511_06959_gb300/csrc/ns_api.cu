@@ -233,10 +233,11 @@ const Coef<float>& bcoef<float>(const ns_ctx* c) { return c->cf; }
 template <>
 const Coef<double>& bcoef<double>(const ns_ctx* c) { return c->cd; }
 
-// W1 (padded, stage type) = w with its ghost layer; the source padded with zero ghosts
+// W1 (padded, stage type) = w with its ghost layer; the source padded with zero ghosts;
+// wpad (may be null): w padded in FP64, the base of a step's last stage
 template <class CT>
-static int bounded_prepare(ns_ctx* c, const double* w, const double* s, const double** sp) {
-  if (ns::launch_bc_embed<CT, double>(c->g, c->bc, 5, 1.0, w, bW<CT>(c, 0), c->st) != cudaSuccess ||
+static int bounded_prepare(ns_ctx* c, const double* w, const double* s, const double** sp, double* wpad = nullptr) {
+  if (ns::launch_bc_embed<CT, double>(c->g, c->bc, 5, 1.0, w, bW<CT>(c, 0), c->st, wpad) != cudaSuccess ||
       ns::launch_bc_ghosts<CT>(c->g, c->bc, bW<CT>(c, 0), c->st) != cudaSuccess)
     return NS_ERR_CUDA;
   *sp = nullptr;
@@ -268,10 +269,8 @@ static int bounded_stage(ns_ctx* c, int i, bool final_out, const double* sp, boo
 template <class CT>
 static int bounded_primal_t(ns_ctx* c, const double* w, const double* s, double* wo) {
   const double* sp = nullptr;
-  int r = bounded_prepare<CT>(c, w, s, &sp);
+  int r = bounded_prepare<CT>(c, w, s, &sp, c->bd[0]);
   if (r) return r;
-  if (ns::launch_bc_embed<double, double>(c->g, c->bc, 5, 1.0, w, c->bd[0], c->st) != cudaSuccess)
-    return NS_ERR_CUDA;
   const Scheme& sc = scheme_of(c);
   for (int i = 0; i < sc.ns; ++i)
     if ((r = bounded_stage<CT>(c, i, true, sp, true))) return r;
@@ -290,10 +289,12 @@ static int bounded_rhs_t(ns_ctx* c, const double* w, const double* s, double* R)
 }
 
 // the transposed product on the padded box of seed sa*A at padded stage state W
-// (into bd[3]), then the boundary epilogue e
+// (into bd[3]), then the boundary epilogue e, which also leaves the next stage's seed in
+// the padded buffer (so only a step's first seed is embedded)
 template <class CT, class NU>
 static int bounded_transposed_stage(ns_ctx* c, const CT* W, ns::BcEpilogue& e, const NU* nu) {
-  if (ns::launch_bc_embed<CT, double>(c->g, c->bc, 5, e.sa, e.A, bW<CT>(c, 5), c->st) != cudaSuccess)
+  if ((e.mode == 0 || e.first) &&
+      ns::launch_bc_embed<CT, double>(c->g, c->bc, 5, e.sa, e.A, bW<CT>(c, 5), c->st) != cudaSuccess)
     return NS_ERR_CUDA;
   ns::AdjArgs<CT, CT, CT> a{};
   a.W = W; a.A = bW<CT>(c, 5); a.ca = 1.0; a.lam_out = c->bd[3];
@@ -302,7 +303,7 @@ static int bounded_transposed_stage(ns_ctx* c, const CT* W, ns::BcEpilogue& e, c
   e.i2[0] = 1.0 / (c->p.dx * c->p.dx);
   e.i2[1] = 1.0 / (c->p.dy * c->p.dy);
   e.i2[2] = 1.0 / (c->p.dz * c->p.dz);
-  return cuerr(ns::launch_bc_adj_epilogue<CT, NU>(c->g, c->bc, e, c->bd[3], W, nu, c->st));
+  return cuerr(ns::launch_bc_adj_epilogue<CT, NU>(c->g, c->bc, e, c->bd[3], W, nu, bW<CT>(c, 5), c->st));
 }
 
 template <class CT>
@@ -501,6 +502,8 @@ int ns_set_boundaries(ns_ctx* c, int bc, const double* far, const double* wall_e
   c->bc.inout = inout;
   c->bc.walls = walls;
   for (int k = 0; k < 5; ++k) c->bc.far[k] = inout ? far[k] : 0.0;
+  c->bc.cf = inout ? sqrt(c->p.gamma * far[4] / far[0]) : 0.0;
+  c->bc.ent = inout ? far[4] / pow(far[0], c->p.gamma) : 0.0;
   for (int k = 0; k < 2; ++k) c->bc.wall_e[k] = walls ? wall_e[k] : 0.0;
   c->gp = c->g;
   c->gp.nx = c->g.nx + 2 * inout;

@@ -11,8 +11,8 @@
 // filled (k_bc_ghosts).  The adjoint is the exact transpose of that map: the periodic
 // transposed product runs on the padded box with a zero adjoint in the ghosts, and
 // k_bc_adj_epilogue pulls each ghost's output back to the cell the ghost was built from
-// through the transposed 5 x 5 ghost Jacobian (forward-mode dual numbers), rows first,
-// then columns (the reverse of the padding's order).  The added adjoint viscosity
+// through the transposed 5 x 5 ghost Jacobian (reversed by hand), rows first, then
+// columns (the reverse of the padding's order).  The added adjoint viscosity
 // passes no flux through the boundary faces, which keeps it symmetric and
 // non-positive; the epilogue applies it on the unpadded box with those faces closed.
 //
@@ -34,14 +34,6 @@ namespace ns {
 
 namespace {
 
-__device__ __forceinline__ Dual dsqrt(Dual a) {
-  const double r = sqrt(a.v);
-  return Dual(r, 0.5 * a.d / r);
-}
-__device__ __forceinline__ Dual dpow(Dual a, double e) {
-  const double r = pow(a.v, e);
-  return Dual(r, e * pow(a.v, e - 1.0) * a.d);
-}
 __device__ __forceinline__ double dsqrt(double a) { return sqrt(a); }
 __device__ __forceinline__ double dpow(double a, double e) { return pow(a, e); }
 __device__ __forceinline__ float dsqrt(float a) { return sqrtf(a); }
@@ -56,8 +48,7 @@ __device__ void char_state(const T wc[5], int side, const BcDesc& bc, T out[5]) 
   const T u0 = wc[1] / rho, u1 = wc[2] / rho, u2 = wc[3] / rho;
   const T p = T(g - 1.0) * (wc[4] - T(0.5) * rho * (u0 * u0 + u1 * u1 + u2 * u2));
   const T c = dsqrt(T(g) * p / rho);
-  const double rf = bc.far[0], uf1 = bc.far[1], uf2 = bc.far[2], uf3 = bc.far[3], pf = bc.far[4];
-  const double cf = sqrt(g * pf / rf);
+  const double uf1 = bc.far[1], uf2 = bc.far[2], uf3 = bc.far[3], cf = bc.cf;
   T Rp, Rm, ent, ut2, ut3;
   if (side == 1) {
     Rp = u0 + T(k) * c;
@@ -68,7 +59,7 @@ __device__ void char_state(const T wc[5], int side, const BcDesc& bc, T out[5]) 
   } else {
     Rp = T(uf1 + k * cf);
     Rm = u0 - T(k) * c;
-    ent = T(pf / pow(rf, g));
+    ent = T(bc.ent);
     ut2 = T(uf2);
     ut3 = T(uf3);
   }
@@ -115,38 +106,48 @@ __device__ __forceinline__ Pad pad_of(const GridDesc& g, const BcDesc& bc) {
   return p;
 }
 
-// padded field (interior copied and converted, ghosts zero), ncomp components per box
+// Row kernels: one warp per row (a component's y-row of one plane), so that the row's
+// place is worked out once per warp and lanes move along x.  (A thread per element spent
+// most of its time on the 64-bit divisions that split its index: 10.3 us for the field of
+// a 96x48x48 duct.)
+constexpr int BR = 8;   // rows (warps) per CTA
+
+// padded fields (interior copied and converted, ghosts zero), ncomp components per box:
+// dst = cvt(scale src); dst2 (may be null) = src unscaled in FP64
 template <class TO, class TI>
-__global__ void k_bc_embed(GridDesc g, BcDesc bc, int ncomp, double scale, const TI* __restrict__ src,
-                           TO* __restrict__ dst) {
+__global__ void __launch_bounds__(32 * BR) k_bc_embed(GridDesc g, BcDesc bc, int ncomp, double scale,
+                                                      const TI* __restrict__ src, TO* __restrict__ dst,
+                                                      double* __restrict__ dst2) {
   const Pad P = pad_of(g, bc);
-  const long long n = P.cellsp * ncomp * g.batch;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const long long bc_ = i / P.cellsp, r = i - bc_ * P.cellsp;
-    const int z = (int)(r / P.planep);
-    const long long rp = r - (long long)z * P.planep;
-    const int yp = (int)(rp / P.nxp), xp = (int)(rp - (long long)yp * P.nxp);
-    const int x = xp - P.ix, y = yp - P.iy;
-    TO v = TO(0);
-    if (x >= 0 && x < g.nx && y >= 0 && y < g.ny) {
-      const double s = (double)src[bc_ * g.cells + (long long)z * g.plane + (long long)y * g.nx + x];
-      v = cvt<TO>(scale * s);
+  const long long rows = (long long)P.nyp * g.nz * ncomp * g.batch;
+  const int lane = threadIdx.x & 31;
+  for (long long r = (long long)blockIdx.x * BR + (threadIdx.x >> 5); r < rows; r += (long long)gridDim.x * BR) {
+    const long long q = r / P.nyp;                       // (box, component, plane)
+    const int y = (int)(r - q * P.nyp) - P.iy;
+    const bool in = y >= 0 && y < g.ny;
+    const TI* s = src + q * g.plane + (long long)(in ? y : 0) * g.nx;
+    TO* d = dst + r * P.nxp;
+    for (int xp = lane; xp < P.nxp; xp += 32) {
+      const int x = xp - P.ix;
+      const double v = in && x >= 0 && x < g.nx ? (double)s[x] : 0.0;
+      d[xp] = cvt<TO>(scale * v);
+      if (dst2) dst2[r * P.nxp + xp] = v;
     }
-    dst[i] = v;
   }
 }
 
 // interior of a padded field
 template <class TO, class TI>
-__global__ void k_bc_crop(GridDesc g, BcDesc bc, int ncomp, const TI* __restrict__ src, TO* __restrict__ dst) {
+__global__ void __launch_bounds__(32 * BR) k_bc_crop(GridDesc g, BcDesc bc, int ncomp, const TI* __restrict__ src,
+                                                     TO* __restrict__ dst) {
   const Pad P = pad_of(g, bc);
-  const long long n = g.cells * ncomp * g.batch;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const long long bc_ = i / g.cells, r = i - bc_ * g.cells;
-    const int z = (int)(r / g.plane);
-    const long long rr = r - (long long)z * g.plane;
-    const int y = (int)(rr / g.nx), x = (int)(rr - (long long)y * g.nx);
-    dst[i] = (TO)src[bc_ * P.cellsp + (long long)z * P.planep + (long long)(y + P.iy) * P.nxp + (x + P.ix)];
+  const long long rows = (long long)g.ny * g.nz * ncomp * g.batch;
+  const int lane = threadIdx.x & 31;
+  for (long long r = (long long)blockIdx.x * BR + (threadIdx.x >> 5); r < rows; r += (long long)gridDim.x * BR) {
+    const long long q = r / g.ny;
+    const int y = (int)(r - q * g.ny);
+    const TI* s = src + q * P.planep + (long long)(y + P.iy) * P.nxp + P.ix;
+    for (int x = lane; x < g.nx; x += 32) dst[r * g.nx + x] = (TO)s[x];
   }
 }
 
@@ -201,24 +202,61 @@ __global__ void k_bc_ghosts(GridDesc g, BcDesc bc, T* __restrict__ W) {
   }
 }
 
-// d = J^T h for the Jacobian J[i][k] = d ghost_i / d wc_k of a characteristic (kind 0)
-// or wall (kind 1) ghost built from wc, by forward-mode dual numbers
-__device__ void ghost_pullback(const double wc[5], int kind, int side, const BcDesc& bc, const double h[5],
-                               double d[5]) {
-#pragma unroll 1
-  for (int k = 0; k < 5; ++k) {
-    Dual x[5], o[5];
+// d = J^T h, J the Jacobian of a wall ghost with respect to the cell wc it was built from:
+// the ghost is (rho, -m, 2 e_w rho - rho E + |m|^2 / rho).
+__device__ __forceinline__ void wall_pullback(const double wc[5], int side, const BcDesc& bc, const double h[5],
+                                              double d[5]) {
+  const double ir = 1.0 / wc[0];
+  const double u[3] = {wc[1] * ir, wc[2] * ir, wc[3] * ir};
+  d[0] = h[0] + h[4] * (2.0 * bc.wall_e[side] - (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]));
 #pragma unroll
-    for (int m = 0; m < 5; ++m) x[m] = Dual(wc[m], m == k ? 1.0 : 0.0);
-    if (kind == 0)
-      char_state<Dual>(x, side, bc, o);
-    else
-      wall_state<Dual>(x, side, bc, o);
-    double acc = 0.0;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) acc += o[i].d * h[i];
-    d[k] = acc;
+  for (int k = 0; k < 3; ++k) d[1 + k] = 2.0 * u[k] * h[4] - h[1 + k];
+  d[4] = -h[4];
+}
+
+// d = J^T h, J the Jacobian of a characteristic ghost with respect to the cell wc it was
+// built from: char_state reversed step by step.  The ghost's density is written
+// rho_b = rho_0 (c_b / c_0)^(2/(gamma-1)), its entropy being that of (rho_0, c_0): the
+// cell's at the outflow, the far field's at the inflow.
+__device__ __forceinline__ void char_pullback(const double wc[5], int side, const BcDesc& bc, const double h[5],
+                                              double d[5]) {
+  const double g = bc.gamma, gm1 = g - 1.0, k = 2.0 / gm1;
+  const double rho = wc[0], ir = 1.0 / rho;
+  const double u[3] = {wc[1] * ir, wc[2] * ir, wc[3] * ir};
+  const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+  const double p = gm1 * (wc[4] - 0.5 * rho * uu);
+  const double c = sqrt(g * p * ir);
+  const bool out = side == 1;
+  const double Rp = out ? u[0] + k * c : bc.far[1] + k * bc.cf;
+  const double Rm = out ? bc.far[1] - k * bc.cf : u[0] - k * c;
+  const double ub = 0.5 * (Rp + Rm), cb = 0.25 * gm1 * (Rp - Rm);
+  const double t2 = out ? u[1] : bc.far[2], t3 = out ? u[2] : bc.far[3];
+  const double r0 = out ? rho : bc.far[0], c0 = out ? c : bc.cf;
+  const double x = cb / c0, x2 = x * x;
+  // (x^2)^(1/(gamma-1)); gamma = 1.4 gives |x|^5
+  const double rb = r0 * (fabs(k - 5.0) < 1e-12 ? x2 * x2 * fabs(x) : pow(x2, 0.5 * k));
+  const double igg = 1.0 / (g * gm1);
+  const double rbb = h[0] + h[1] * ub + h[2] * t2 + h[3] * t3 +
+                     h[4] * (cb * cb * igg + 0.5 * (ub * ub + t2 * t2 + t3 * t3));
+  const double ubb = rb * (h[1] + h[4] * ub);
+  const double krb = k * rb * rbb;
+  const double cbb = 2.0 * h[4] * rb * cb * igg + krb / cb;
+  const double Rb = out ? 0.5 * ubb + 0.25 * gm1 * cbb : 0.5 * ubb - 0.25 * gm1 * cbb;
+  double us[3] = {Rb, 0.0, 0.0}, rs = 0.0;
+  double cs = out ? k * Rb : -k * Rb;
+  if (out) {
+    us[1] = rb * (h[2] + h[4] * t2);
+    us[2] = rb * (h[3] + h[4] * t3);
+    rs = rbb * rb * ir;
+    cs -= krb / c;
   }
+  // c^2 = gamma p / rho, then (rho, u, p) to conservative variables
+  const double ps = cs * c / (2.0 * p);
+  rs -= 0.5 * cs * c * ir;
+  d[0] = rs - (us[0] * u[0] + us[1] * u[1] + us[2] * u[2]) * ir + 0.5 * gm1 * uu * ps;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) d[1 + j] = us[j] * ir - gm1 * u[j] * ps;
+  d[4] = gm1 * ps;
 }
 
 // The boundary epilogue of one transposed stage on a bounded box, per interior cell:
@@ -227,125 +265,171 @@ __device__ void ghost_pullback(const double wc[5], int kind, int side, const BcD
 //   mode 0 (transposed residual only):  out = g
 //   mode 1 (a Runge-Kutta stage):        Gs = (first ? 0 : G) + g; G = Gs (not last);
 //       a_next = cl lam + cg g + cs Gs (not last); lam_out = lam + Gs (last);
-//       sbar += a (when sbar != null)
+//       sbar += a (when sbar != null); seed = a_next in the padded stage type, the next
+//       stage's input (its ghosts stay zero)
 // gp: the transposed product on the padded box (FP64); W: the padded stage state
 // (ghost inputs); A, sa: the stage's seed a = sa A (unpadded FP64).
+//
+// The pull-backs take a few hundred FP64 instructions, which GB300 issues at 1/64 of the
+// FP32 rate, and only the cells next to a boundary need them: the first nbb CTAs take
+// those cells, packed so that all 32 lanes of a warp have one, and the other CTAs the
+// cells of whole rows, leaving out the packed ones.  With every cell in one grid, each
+// row's end cells held two of its three warps for the whole pull-back: 931 us per stage of
+// a 96x48x48 duct (a primal and an adjoint step: 4080 us, now 720 us).
+struct EpiArgs {
+  const double* gp;
+  const double* A;
+  double sa, nus[3], i2[3];
+  int mode, first, last;
+  const double* lam;
+  double* G;
+  double cl, cg, cs;
+  double* a_next;
+  double* out;
+  double* sbar;
+};
+
 template <class CT, class NU>
-__global__ void k_bc_adj_epilogue(GridDesc g, BcDesc bc, const double* __restrict__ gp, const CT* __restrict__ W,
-                                  const double* __restrict__ A, double sa, const NU* __restrict__ nu, double nus0,
-                                  double nus1, double nus2, double i2x, double i2y, double i2z, int mode, int first,
-                                  int last, const double* __restrict__ lam, double* __restrict__ G, double cl,
-                                  double cg, double cs, double* __restrict__ a_next, double* __restrict__ out,
-                                  double* __restrict__ sbar) {
-  const Pad P = pad_of(g, bc);
-  const long long n = g.cells * g.batch;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const long long b = i / g.cells, r = i - b * g.cells;
-    const int z = (int)(r / g.plane);
-    const long long rr = r - (long long)z * g.plane;
-    const int y = (int)(rr / g.nx), x = (int)(rr - (long long)y * g.nx);
-    const long long boxp = b * 5 * P.cellsp + (long long)z * P.planep;
-    auto atp = [&](int xp, int yp) { return boxp + (long long)yp * P.nxp + xp; };
-    auto wget = [&](long long o, double v[5]) {
+__device__ __forceinline__ void epilogue_cell(const GridDesc& g, const Pad& P, const EpiArgs& e,
+                                              const NU* __restrict__ nu, CT* __restrict__ seed, int b, int x, int y,
+                                              int z, double gc[5]) {
+  const long long r = (long long)z * g.plane + (long long)y * g.nx + x;
+  const long long o = (long long)b * 5 * g.cells + r;
+  const double sa = e.sa;
+  double a[5];
 #pragma unroll
-      for (int k = 0; k < 5; ++k) v[k] = (double)W[o + k * P.cellsp];
-    };
-    auto gget = [&](long long o, double v[5]) {
-#pragma unroll
-      for (int k = 0; k < 5; ++k) v[k] = gp[o + k * P.cellsp];
-    };
-    const int xp = x + P.ix, yp = y + P.iy;
-    double gc[5], h[5], d[5], wc[5];
-    gget(atp(xp, yp), gc);
-    // wall rows first: a ghost row's output goes to the row it was built from
-    if (P.iy && (y == 0 || y == g.ny - 1)) {
-      for (int side = 0; side < 2; ++side) {
-        if ((side == 0 && y != 0) || (side == 1 && y != g.ny - 1)) continue;
-        gget(atp(xp, side == 0 ? 0 : P.nyp - 1), h);
-        wget(atp(xp, yp), wc);
-        ghost_pullback(wc, 1, side, bc, h, d);
-#pragma unroll
-        for (int k = 0; k < 5; ++k) gc[k] += d[k];
-      }
-    }
-    // then the inflow and outflow columns: each column ghost's output, with its wall
-    // ghosts' outputs pulled back onto it at the first and last rows
-    if (P.ix && (x == 0 || x == g.nx - 1)) {
-      for (int side = 0; side < 2; ++side) {
-        if ((side == 0 && x != 0) || (side == 1 && x != g.nx - 1)) continue;
-        const int xg = side == 0 ? 0 : P.nxp - 1;
-        gget(atp(xg, yp), h);
-        if (P.iy && (y == 0 || y == g.ny - 1)) {
-          for (int ws = 0; ws < 2; ++ws) {
-            if ((ws == 0 && y != 0) || (ws == 1 && y != g.ny - 1)) continue;
-            double hc[5], dc[5], wg[5];
-            gget(atp(xg, ws == 0 ? 0 : P.nyp - 1), hc);
-            wget(atp(xg, yp), wg);   // the column ghost the corner was built from
-            ghost_pullback(wg, 1, ws, bc, hc, dc);
-#pragma unroll
-            for (int k = 0; k < 5; ++k) h[k] += dc[k];
-          }
-        }
-        wget(atp(xp, yp), wc);
-        ghost_pullback(wc, 0, side, bc, h, d);
-#pragma unroll
-        for (int k = 0; k < 5; ++k) gc[k] += d[k];
-      }
-    }
-    // the seed of this stage and the added viscosity with closed boundary faces
-    const long long o = b * 5 * g.cells + r;
-    double a[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) a[k] = sa * A[o + k * g.cells];
-    if (nu) {
-      const long long c0 = b * g.cells + r;
-      const double nc = (double)nu[c0];
-      const int xm = x == 0 ? g.nx - 1 : x - 1, xq = x == g.nx - 1 ? 0 : x + 1;
-      const int ym = y == 0 ? g.ny - 1 : y - 1, yq = y == g.ny - 1 ? 0 : y + 1;
-      const int zm = z == 0 ? g.nz - 1 : z - 1, zq = z == g.nz - 1 ? 0 : z + 1;
-      const bool cxm = P.ix && x == 0, cxq = P.ix && x == g.nx - 1;   // closed faces
-      const bool cym = P.iy && y == 0, cyq = P.iy && y == g.ny - 1;
-      const long long bb = b * g.cells;
-      const long long oxm = (long long)z * g.plane + (long long)y * g.nx + xm;
-      const long long oxq = (long long)z * g.plane + (long long)y * g.nx + xq;
-      const long long oym = (long long)z * g.plane + (long long)ym * g.nx + x;
-      const long long oyq = (long long)z * g.plane + (long long)yq * g.nx + x;
-      const long long ozm = (long long)zm * g.plane + (long long)y * g.nx + x;
-      const long long ozq = (long long)zq * g.plane + (long long)y * g.nx + x;
-      const double fxm = cxm ? 0.0 : 0.5 * (nc + (double)nu[bb + oxm]);
-      const double fxq = cxq ? 0.0 : 0.5 * (nc + (double)nu[bb + oxq]);
-      const double fym = cym ? 0.0 : 0.5 * (nc + (double)nu[bb + oym]);
-      const double fyq = cyq ? 0.0 : 0.5 * (nc + (double)nu[bb + oyq]);
-      const double fzm = 0.5 * (nc + (double)nu[bb + ozm]);
-      const double fzq = 0.5 * (nc + (double)nu[bb + ozq]);
-      const long long ab = b * 5 * g.cells;
-#pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        const double* Ak = A + ab + (long long)k * g.cells;
-        const double ac = a[k];
-        const double L = (fxq * (sa * Ak[oxq] - ac) - fxm * (ac - sa * Ak[oxm])) * i2x +
-                         (fyq * (sa * Ak[oyq] - ac) - fym * (ac - sa * Ak[oym])) * i2y +
-                         (fzq * (sa * Ak[ozq] - ac) - fzm * (ac - sa * Ak[ozm])) * i2z;
-        gc[k] += (k == 0 ? nus0 : (k == 4 ? nus2 : nus1)) * L;
-      }
-    }
+  for (int k = 0; k < 5; ++k) a[k] = sa * e.A[o + k * g.cells];
+  if (nu) {
+    const NU* nb = nu + (long long)b * g.cells;
+    const double nc = (double)nb[r];
+    const long long oxm = r + (x == 0 ? g.nx - 1 : -1), oxq = r + (x == g.nx - 1 ? 1 - g.nx : 1);
+    const long long oym = r + (long long)(y == 0 ? g.ny - 1 : -1) * g.nx,
+                    oyq = r + (long long)(y == g.ny - 1 ? 1 - g.ny : 1) * g.nx;
+    const long long ozm = r + (z == 0 ? g.nz - 1 : -1) * g.plane, ozq = r + (z == g.nz - 1 ? 1 - g.nz : 1) * g.plane;
+    // closed faces pass nothing
+    const double fxm = P.ix && x == 0 ? 0.0 : 0.5 * (nc + (double)nb[oxm]);
+    const double fxq = P.ix && x == g.nx - 1 ? 0.0 : 0.5 * (nc + (double)nb[oxq]);
+    const double fym = P.iy && y == 0 ? 0.0 : 0.5 * (nc + (double)nb[oym]);
+    const double fyq = P.iy && y == g.ny - 1 ? 0.0 : 0.5 * (nc + (double)nb[oyq]);
+    const double fzm = 0.5 * (nc + (double)nb[ozm]), fzq = 0.5 * (nc + (double)nb[ozq]);
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      const long long ok = o + (long long)k * g.cells;
-      if (mode == 0) {
-        out[ok] = gc[k];
-        continue;
-      }
-      const double Gs = (first ? 0.0 : G[ok]) + gc[k];
-      if (last) {
-        out[ok] = lam[ok] + Gs;
-      } else {
-        G[ok] = Gs;
-        a_next[ok] = cl * lam[ok] + cg * gc[k] + cs * Gs;
-      }
-      if (sbar) sbar[ok] += a[k];
+      const double* Ak = e.A + (long long)b * 5 * g.cells + (long long)k * g.cells;
+      const double ac = a[k];
+      const double L = (fxq * (sa * Ak[oxq] - ac) - fxm * (ac - sa * Ak[oxm])) * e.i2[0] +
+                       (fyq * (sa * Ak[oyq] - ac) - fym * (ac - sa * Ak[oym])) * e.i2[1] +
+                       (fzq * (sa * Ak[ozq] - ac) - fzm * (ac - sa * Ak[ozm])) * e.i2[2];
+      gc[k] += e.nus[k == 0 ? 0 : (k == 4 ? 2 : 1)] * L;
     }
   }
+  const long long op = (long long)b * 5 * P.cellsp + (long long)z * P.planep + (long long)(y + P.iy) * P.nxp + x + P.ix;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const long long ok = o + (long long)k * g.cells;
+    if (e.mode == 0) {
+      e.out[ok] = gc[k];
+      continue;
+    }
+    const double Gs = (e.first ? 0.0 : e.G[ok]) + gc[k];
+    if (e.last) {
+      e.out[ok] = e.lam[ok] + Gs;
+    } else {
+      e.G[ok] = Gs;
+      const double an = e.cl * e.lam[ok] + e.cg * gc[k] + e.cs * Gs;
+      e.a_next[ok] = an;
+      seed[op + (long long)k * P.cellsp] = cvt<CT>(an);
+    }
+    if (e.sbar) e.sbar[ok] += a[k];
+  }
+}
+
+constexpr int BBT = 32;   // packed boundary cells per CTA: one warp, so that they spread over the SMs
+
+template <class CT, class NU>
+__global__ void __launch_bounds__(32 * BR) k_bc_adj_epilogue(GridDesc g, BcDesc bc, EpiArgs e,
+                                                             const CT* __restrict__ W, const NU* __restrict__ nu,
+                                                             CT* __restrict__ seed, int nbb) {
+  const Pad P = pad_of(g, bc);
+  const int lane = threadIdx.x & 31;
+  if ((int)blockIdx.x >= nbb) {
+    // whole rows, without the cells next to a boundary
+    const long long rows = (long long)g.ny * g.nz * g.batch, step = (long long)(gridDim.x - nbb) * BR;
+    for (long long r = (long long)(blockIdx.x - nbb) * BR + (threadIdx.x >> 5); r < rows; r += step) {
+      const int y = (int)(r % g.ny);
+      const long long q = r / g.ny;
+      const int z = (int)(q % g.nz), b = (int)(q / g.nz);
+      if (P.iy && (y == 0 || y == g.ny - 1)) continue;
+      const double* gr = e.gp + (long long)b * 5 * P.cellsp + (long long)z * P.planep +
+                         (long long)(y + P.iy) * P.nxp + P.ix;
+      for (int x = lane; x < g.nx; x += 32) {
+        if (P.ix && (x == 0 || x == g.nx - 1)) continue;
+        double gc[5];
+        load5(gr, x, P.cellsp, gc);
+        epilogue_cell<CT, NU>(g, P, e, nu, seed, b, x, y, z, gc);
+      }
+    }
+    return;
+  }
+  if (threadIdx.x >= BBT) return;
+  // cells next to a boundary of one plane: the inflow and outflow columns (an only column
+  // is both), then the wall rows without the columns' cells
+  const int ncol = P.ix ? (g.nx > 1 ? 2 : 1) : 0, nrow = P.iy ? (g.ny > 1 ? 2 : 1) : 0;
+  const int rw = g.nx - ncol;                            // cells of a wall row outside the columns
+  const int per = ncol * g.ny + nrow * rw;
+  const long long i = (long long)blockIdx.x * BBT + threadIdx.x;
+  if (i >= (long long)per * g.nz * g.batch) return;
+  const long long q = i / per;
+  const int z = (int)(q % g.nz), b = (int)(q / g.nz);
+  int j = (int)(i - q * per), x, y;
+  if (j < ncol * g.ny) {
+    x = j < g.ny ? 0 : g.nx - 1;
+    y = j < g.ny ? j : j - g.ny;
+  } else {
+    j -= ncol * g.ny;
+    y = j < rw ? 0 : g.ny - 1;
+    x = (j < rw ? j : j - rw) + (P.ix ? 1 : 0);
+  }
+  const long long boxp = (long long)b * 5 * P.cellsp + (long long)z * P.planep;
+  auto atp = [&](int xp, int yp) { return boxp + (long long)yp * P.nxp + xp; };
+  auto wget = [&](long long o, double v[5]) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) v[k] = (double)W[o + k * P.cellsp];
+  };
+  const int xp = x + P.ix, yp = y + P.iy;
+  double gc[5], h[5], d[5], wc[5];
+  load5(e.gp, atp(xp, yp), P.cellsp, gc);
+  wget(atp(xp, yp), wc);
+  // wall rows first: a ghost row's output goes to the row it was built from
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    if (!P.iy || y != (side == 0 ? 0 : g.ny - 1)) continue;
+    load5(e.gp, atp(xp, side == 0 ? 0 : P.nyp - 1), P.cellsp, h);
+    wall_pullback(wc, side, bc, h, d);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) gc[k] += d[k];
+  }
+  // then the inflow and outflow columns: each column ghost's output, with its wall
+  // ghosts' outputs pulled back onto it at the first and last rows
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    if (!P.ix || x != (side == 0 ? 0 : g.nx - 1)) continue;
+    const int xg = side == 0 ? 0 : P.nxp - 1;
+    load5(e.gp, atp(xg, yp), P.cellsp, h);
+#pragma unroll 1
+    for (int ws = 0; ws < 2; ++ws) {
+      if (!P.iy || y != (ws == 0 ? 0 : g.ny - 1)) continue;
+      double hc[5], wg[5];
+      load5(e.gp, atp(xg, ws == 0 ? 0 : P.nyp - 1), P.cellsp, hc);
+      wget(atp(xg, yp), wg);   // the column ghost the corner was built from
+      wall_pullback(wg, ws, bc, hc, d);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) h[k] += d[k];
+    }
+    char_pullback(wc, side, bc, h, d);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) gc[k] += d[k];
+  }
+  epilogue_cell<CT, NU>(g, P, e, nu, seed, b, x, y, z, gc);
 }
 
 constexpr int BB = 256;
@@ -362,19 +446,25 @@ long long bc_padded_cells(const GridDesc& g, const BcDesc& bc) {
   return (long long)(g.nx + 2 * bc.inout) * (g.ny + 2 * bc.walls) * g.nz;
 }
 
+// CTAs of the row kernels: BR rows each, at most sixteen per SM (the rest by the stride)
+static unsigned blocks_for_rows(long long rows) {
+  const long long b = (rows + BR - 1) / BR;
+  return (unsigned)(b < 152 * 16 ? (b > 0 ? b : 1) : 152 * 16);
+}
+
 template <class TO, class TI>
 cudaError_t launch_bc_embed(const GridDesc& g, const BcDesc& bc, int ncomp, double scale, const TI* src, TO* dst,
-                            cudaStream_t st) {
-  const long long n = bc_padded_cells(g, bc) * ncomp * g.batch;
-  k_bc_embed<TO, TI><<<blocks_for(n), BB, 0, st>>>(g, bc, ncomp, scale, src, dst);
+                            cudaStream_t st, double* dst2) {
+  const long long rows = (long long)(g.ny + 2 * bc.walls) * g.nz * ncomp * g.batch;
+  k_bc_embed<TO, TI><<<blocks_for_rows(rows), 32 * BR, 0, st>>>(g, bc, ncomp, scale, src, dst, dst2);
   count_launch();
   return cudaGetLastError();
 }
 
 template <class TO, class TI>
 cudaError_t launch_bc_crop(const GridDesc& g, const BcDesc& bc, int ncomp, const TI* src, TO* dst, cudaStream_t st) {
-  const long long n = g.cells * ncomp * g.batch;
-  k_bc_crop<TO, TI><<<blocks_for(n), BB, 0, st>>>(g, bc, ncomp, src, dst);
+  const long long rows = (long long)g.ny * g.nz * ncomp * g.batch;
+  k_bc_crop<TO, TI><<<blocks_for_rows(rows), 32 * BR, 0, st>>>(g, bc, ncomp, src, dst);
   count_launch();
   return cudaGetLastError();
 }
@@ -389,18 +479,27 @@ cudaError_t launch_bc_ghosts(const GridDesc& g, const BcDesc& bc, T* W, cudaStre
 
 template <class CT, class NU>
 cudaError_t launch_bc_adj_epilogue(const GridDesc& g, const BcDesc& bc, const BcEpilogue& e, const double* gp,
-                                   const CT* W, const NU* nu, cudaStream_t st) {
-  k_bc_adj_epilogue<CT, NU><<<blocks_for(g.cells * g.batch), BB, 0, st>>>(
-      g, bc, gp, W, e.A, e.sa, nu, e.nus[0], e.nus[1], e.nus[2], e.i2[0], e.i2[1], e.i2[2], e.mode, e.first, e.last,
-      e.lam, e.G, e.cl, e.cg, e.cs, e.a_next, e.out, e.sbar);
+                                   const CT* W, const NU* nu, CT* seed, cudaStream_t st) {
+  EpiArgs a;
+  a.gp = gp; a.A = e.A; a.sa = e.sa;
+  for (int k = 0; k < 3; ++k) { a.nus[k] = e.nus[k]; a.i2[k] = e.i2[k]; }
+  a.mode = e.mode; a.first = e.first; a.last = e.last;
+  a.lam = e.lam; a.G = e.G; a.cl = e.cl; a.cg = e.cg; a.cs = e.cs;
+  a.a_next = e.a_next; a.out = e.out; a.sbar = e.sbar;
+  const long long ncol = bc.inout ? (g.nx > 1 ? 2 : 1) : 0, nrow = bc.walls ? (g.ny > 1 ? 2 : 1) : 0;
+  const long long cells = (ncol * g.ny + nrow * (g.nx - ncol)) * g.nz * g.batch;   // next to a boundary
+  const long long nbb = (cells + BBT - 1) / BBT;
+  if (nbb > (1LL << 30)) return cudaErrorInvalidConfiguration;
+  const unsigned rows = blocks_for_rows((long long)g.ny * g.nz * g.batch);
+  k_bc_adj_epilogue<CT, NU><<<(unsigned)nbb + rows, 32 * BR, 0, st>>>(g, bc, a, W, nu, seed, (int)nbb);
   count_launch();
   return cudaGetLastError();
 }
 
 template cudaError_t launch_bc_embed<double, double>(const GridDesc&, const BcDesc&, int, double, const double*,
-                                                     double*, cudaStream_t);
+                                                     double*, cudaStream_t, double*);
 template cudaError_t launch_bc_embed<float, double>(const GridDesc&, const BcDesc&, int, double, const double*,
-                                                    float*, cudaStream_t);
+                                                    float*, cudaStream_t, double*);
 template cudaError_t launch_bc_crop<double, double>(const GridDesc&, const BcDesc&, int, const double*, double*,
                                                     cudaStream_t);
 template cudaError_t launch_bc_crop<float, float>(const GridDesc&, const BcDesc&, int, const float*, float*,
@@ -408,10 +507,10 @@ template cudaError_t launch_bc_crop<float, float>(const GridDesc&, const BcDesc&
 template cudaError_t launch_bc_ghosts<double>(const GridDesc&, const BcDesc&, double*, cudaStream_t);
 template cudaError_t launch_bc_ghosts<float>(const GridDesc&, const BcDesc&, float*, cudaStream_t);
 template cudaError_t launch_bc_adj_epilogue<double, float>(const GridDesc&, const BcDesc&, const BcEpilogue&,
-                                                           const double*, const double*, const float*, cudaStream_t);
+                                                           const double*, const double*, const float*, double*, cudaStream_t);
 template cudaError_t launch_bc_adj_epilogue<double, double>(const GridDesc&, const BcDesc&, const BcEpilogue&,
-                                                            const double*, const double*, const double*, cudaStream_t);
+                                                            const double*, const double*, const double*, double*, cudaStream_t);
 template cudaError_t launch_bc_adj_epilogue<float, float>(const GridDesc&, const BcDesc&, const BcEpilogue&,
-                                                          const double*, const float*, const float*, cudaStream_t);
+                                                          const double*, const float*, const float*, float*, cudaStream_t);
 
 }  // namespace ns

@@ -147,6 +147,7 @@ struct BcDesc {
   int walls;          // 1: isothermal no-slip walls at y = 0 and y = L_y
   double gamma;
   double far[5];      // far-field primitive state (rho, u1, u2, u3, p)
+  double cf, ent;     // its sound speed and its entropy p / rho^gamma
   double wall_e[2];   // internal energy e = c_v T of the bottom and the top wall
 };
 // one transposed stage's boundary epilogue (see k_bc_adj_epilogue)
@@ -166,13 +167,13 @@ struct BcEpilogue {
 long long bc_padded_cells(const GridDesc& g, const BcDesc& bc);
 template <class TO, class TI>
 cudaError_t launch_bc_embed(const GridDesc& g, const BcDesc& bc, int ncomp, double scale, const TI* src, TO* dst,
-                            cudaStream_t st);
+                            cudaStream_t st, double* dst2 = nullptr);
 template <class TO, class TI>
 cudaError_t launch_bc_crop(const GridDesc& g, const BcDesc& bc, int ncomp, const TI* src, TO* dst, cudaStream_t st);
 template <class T>
 cudaError_t launch_bc_ghosts(const GridDesc& g, const BcDesc& bc, T* W, cudaStream_t st);
 template <class CT, class NU>
 cudaError_t launch_bc_adj_epilogue(const GridDesc& g, const BcDesc& bc, const BcEpilogue& e, const double* gp,
-                                   const CT* W, const NU* nu, cudaStream_t st);
+                                   const CT* W, const NU* nu, CT* seed, cudaStream_t st);
 
 }  // namespace ns
