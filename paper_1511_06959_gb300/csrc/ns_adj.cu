@@ -125,17 +125,17 @@ __device__ __forceinline__ void adj_plane_store(const AdjPlaneRegs<CT>& r, CT* _
 }
 
 // s-vector of the face between shared positions iL (slot of QL/AL) and iR.
-template <int D, class CT>
+template <int D, int SPT = SP, class CT>
 __device__ __forceinline__ void face_s(const Coef<CT>& c, const CT* QL, const CT* AL, int iL,
                                        const CT* QR, const CT* AR, int iR, CT s[3], CT& fb4) {
-  fb4 = (AL[4 * SP + iL] - AR[4 * SP + iR]) * c.idx[D];
+  fb4 = (AL[4 * SPT + iL] - AR[4 * SPT + iR]) * c.idx[D];
   int j0 = 0;
   if constexpr (std::is_same<CT, float>::value) {
     // components 1 and 2 side by side in paired FP32 instructions
-    const float2 fb = __fmul2_rn(sub2(f2(AL[SP + iL], AL[2 * SP + iL]), f2(AR[SP + iR], AR[2 * SP + iR])),
+    const float2 fb = __fmul2_rn(sub2(f2(AL[SPT + iL], AL[2 * SPT + iL]), f2(AR[SPT + iR], AR[2 * SPT + iR])),
                                  f2(c.idx[D], c.idx[D]));
     const float2 uf = __fmul2_rn(f2(0.5f, 0.5f),
-                                 __fadd2_rn(f2(QL[SP + iL], QL[2 * SP + iL]), f2(QR[SP + iR], QR[2 * SP + iR])));
+                                 __fadd2_rn(f2(QL[SPT + iL], QL[2 * SPT + iL]), f2(QR[SPT + iR], QR[2 * SPT + iR])));
     const float2 sv = __ffma2_rn(f2(fb4, fb4), uf, fb);
     s[0] = sv.x;
     s[1] = sv.y;
@@ -143,8 +143,8 @@ __device__ __forceinline__ void face_s(const Coef<CT>& c, const CT* QL, const CT
   }
 #pragma unroll
   for (int j = j0; j < 3; ++j) {
-    const CT fb = (AL[(1 + j) * SP + iL] - AR[(1 + j) * SP + iR]) * c.idx[D];
-    const CT uf = CT(0.5) * (QL[(1 + j) * SP + iL] + QR[(1 + j) * SP + iR]);
+    const CT fb = (AL[(1 + j) * SPT + iL] - AR[(1 + j) * SPT + iR]) * c.idx[D];
+    const CT uf = CT(0.5) * (QL[(1 + j) * SPT + iL] + QR[(1 + j) * SPT + iR]);
     s[j] = fb + fb4 * uf;
   }
 }
@@ -170,15 +170,15 @@ __device__ __forceinline__ void face_stress(const Coef<CT>& c, const CT* qL, con
 }
 
 // 7-value packet of a face from its s-vector and Fb[4]: nb[0..2] (u), nb[3] (e), ub[0..2].
-template <int D, class CT>
+template <int D, int SPT = SP, class CT>
 __device__ __forceinline__ void face_packet_s(const Coef<CT>& c, const CT s[3], CT fb4, const CT* QL,
                                               int iL, const CT* QR, int iR, const CT* gt1,
                                               const CT* gt2, CT pk[7]) {
   CT uL[3], uR[3], sig[3];
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    uL[j] = QL[(1 + j) * SP + iL];
-    uR[j] = QR[(1 + j) * SP + iR];
+    uL[j] = QL[(1 + j) * SPT + iL];
+    uR[j] = QR[(1 + j) * SPT + iR];
   }
   face_stress<D>(c, uL, uR, gt1, gt2, sig);
 #pragma unroll
@@ -187,15 +187,6 @@ __device__ __forceinline__ void face_packet_s(const Coef<CT>& c, const CT s[3], 
   pk[3] = c.alpha * fb4;
 #pragma unroll
   for (int j = 0; j < 3; ++j) pk[4 + j] = fb4 * sig[j];
-}
-
-template <int D, class CT>
-__device__ __forceinline__ void face_packet(const Coef<CT>& c, const CT* QL, const CT* AL, int iL,
-                                            const CT* QR, const CT* AR, int iR, const CT* gt1,
-                                            const CT* gt2, CT pk[7]) {
-  CT s[3], fb4;
-  face_s<D>(c, QL, AL, iL, QR, AR, iR, s, fb4);
-  face_packet_s<D>(c, s, fb4, QL, iL, QR, iR, gt1, gt2, pk);
 }
 
 // In-plane face values of one plane slot, each face once: s-vector and Fb[4] of the
@@ -363,15 +354,15 @@ __device__ __forceinline__ void zpacket(const CT* sQ, const Coef<CT>& c, int sL,
 // Roe part of a face packet: the adjoints of the two cells' primitives from the Roe
 // dissipation, pk[0..4] for the left cell and pk[5..9] for the right cell, for the
 // face adjoint Db = (a_L - a_R) / dx_D (D enters the face flux with the sign of F^v).
-template <int D, class CT>
+template <int D, int SPT = SP, class CT>
 __device__ __forceinline__ void roe_packet(const Coef<CT>& c, const CT* QL, const CT* AL, int iL,
                                            const CT* QR, const CT* AR, int iR, CT* pk) {
   CT qL[5], qR[5], Db[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
-    qL[v] = QL[v * SP + iL];
-    qR[v] = QR[v * SP + iR];
-    Db[v] = (AL[v * SP + iL] - AR[v * SP + iR]) * c.idx[D];
+    qL[v] = QL[v * SPT + iL];
+    qR[v] = QR[v * SPT + iR];
+    Db[v] = (AL[v * SPT + iL] - AR[v * SPT + iR]) * c.idx[D];
   }
   roe_dissipation_adj<D>(c, qL, qR, Db, pk, pk + 5);
 }
@@ -418,6 +409,182 @@ __device__ __forceinline__ void fill_Z(CT* __restrict__ Z, const CT* __restrict_
 template <class CT, bool ROE> struct AdjMinBlocks { static constexpr int value = NT >= 256 ? 1 : 2; };
 template <> struct AdjMinBlocks<float, false> { static constexpr int value = 512 / NT; };
 template <> struct AdjMinBlocks<float, true> { static constexpr int value = NT >= 256 ? 1 : 3; };
+
+// Convective part of the product at one cell, from the viscous primitive adjoints qb, and
+// its pull-back to conservative variables.  Q: primitives (component stride SPT), ic: the cell.
+template <class CT, int SPT>
+struct Convective {
+  CT rho, u[3], e, ir, Esp, H, rb, mb[3], Eb, pb, ub[3], eb;   // H = rho E + p
+  __device__ __forceinline__ Convective(const Coef<CT>& c, const CT* Q, int ic, const CT qb[4]) {
+    rho = Q[ic];
+    u[0] = Q[SPT + ic];
+    u[1] = Q[2 * SPT + ic];
+    u[2] = Q[3 * SPT + ic];
+    e = Q[4 * SPT + ic];
+    ir = CT(1) / rho;
+    Esp = e + CT(0.5) * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);   // rho E / rho
+    // written out so that every kernel rounds it alike
+    if constexpr (std::is_same<CT, float>::value) H = __fmaf_rn(__fmul_rn(c.gm1, rho), e, __fmul_rn(rho, Esp));
+    else H = rho * Esp + c.gm1 * rho * e;
+    rb = CT(0);
+    Eb = CT(0);
+    pb = CT(0);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      mb[j] = CT(0);
+      ub[j] = qb[j];
+    }
+    eb = qb[3];
+  }
+  // adjoints of (rho, u, e) from the Roe dissipation
+  __device__ __forceinline__ void add_roe(const CT rs[5]) {
+    rb = rs[0];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) ub[j] = ub[j] + rs[1 + j];
+    eb = eb + rs[4];
+  }
+  // F = (a(c + e_D) - a(c - e_D)) / (2 dx_D)
+  template <int D>
+  __device__ __forceinline__ void direction(const CT F[5]) {
+    const CT md = rho * u[D];
+    mb[D] = mb[D] + F[0] + F[1] * u[0] + F[2] * u[1] + F[3] * u[2];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) ub[j] = ub[j] + F[1 + j] * md;
+    pb = pb + F[1 + D] + F[4] * u[D];
+    Eb = Eb + F[4] * u[D];
+    ub[D] = ub[D] + F[4] * H;
+  }
+  __device__ __forceinline__ void pull_back(const Coef<CT>& c, CT gout[5]) {
+    rb = rb + c.gm1 * e * pb;
+    eb = eb + c.gm1 * rho * pb;
+    Eb = Eb + eb * ir;
+    rb = rb - eb * Esp * ir;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      ub[j] = ub[j] - eb * u[j];
+      mb[j] = mb[j] + ub[j] * ir;
+      rb = rb - ub[j] * u[j] * ir;
+    }
+    gout[0] = rb;
+    gout[1] = mb[0];
+    gout[2] = mb[1];
+    gout[3] = mb[2];
+    gout[4] = Eb;
+  }
+};
+
+// Added adjoint viscosity L_nu a at one cell, times the factor of the component's state
+// variable (rho, rho u, rho E).  A0: the plane's adjoint input (component stride SPT), Ap
+// the plane above, am the cell's values in the plane below; n*: nu at the cell and its
+// neighbours.  Z = false leaves out the z-direction (2D boxes).
+template <int SPT, bool Z, class CT>
+__device__ __forceinline__ void add_viscosity(const Coef<CT>& c, const double nus[3], const CT* A0, const CT* Ap,
+                                              const CT* am, int ic, CT nc, CT nxm, CT nxp, CT nym, CT nyp, CT nzm,
+                                              CT nzp, CT gout[5]) {
+  const CT h = CT(0.5);
+  const CT ix2 = c.idx[0] * c.idx[0], iy2 = c.idx[1] * c.idx[1], iz2 = c.idx[2] * c.idx[2];
+  int v0 = 0;
+  if constexpr (std::is_same<CT, float>::value) {
+    // components (0, 1) and (2, 3) side by side in paired FP32 instructions
+    const float2 fxp = f2(h * (nc + nxp), h * (nc + nxp)), fxm = f2(-h * (nc + nxm), -h * (nc + nxm));
+    const float2 fyp = f2(h * (nc + nyp), h * (nc + nyp)), fym = f2(-h * (nc + nym), -h * (nc + nym));
+    const float2 fzp = f2(h * (nc + nzp), h * (nc + nzp)), fzm = f2(-h * (nc + nzm), -h * (nc + nzm));
+#pragma unroll
+    for (int v = 0; v < 4; v += 2) {
+      const float* Av = A0 + v * SPT;
+      const float* Aw = Av + SPT;
+      const float2 ac = f2(Av[ic], Aw[ic]);
+      const float2 tx = __ffma2_rn(fxp, sub2(f2(Av[ic + 1], Aw[ic + 1]), ac),
+                                   __fmul2_rn(fxm, sub2(ac, f2(Av[ic - 1], Aw[ic - 1]))));
+      const float2 ty = __ffma2_rn(fyp, sub2(f2(Av[ic + SX], Aw[ic + SX]), ac),
+                                   __fmul2_rn(fym, sub2(ac, f2(Av[ic - SX], Aw[ic - SX]))));
+      float2 L = __ffma2_rn(ty, f2(iy2, iy2), __fmul2_rn(tx, f2(ix2, ix2)));
+      if constexpr (Z) {
+        const float2 tz = __ffma2_rn(fzp, sub2(f2(Ap[v * SPT + ic], Ap[(v + 1) * SPT + ic]), ac),
+                                     __fmul2_rn(fzm, sub2(ac, f2(am[v], am[v + 1]))));
+        L = __ffma2_rn(tz, f2(iz2, iz2), L);
+      }
+      const float2 gv = __ffma2_rn(f2(float(nus[v == 0 ? 0 : 1]), float(nus[1])), L, f2(gout[v], gout[v + 1]));
+      gout[v] = gv.x;
+      gout[v + 1] = gv.y;
+    }
+    v0 = 4;
+  }
+#pragma unroll
+  for (int v = v0; v < 5; ++v) {
+    const CT* Av = A0 + v * SPT;
+    const CT ac = Av[ic];
+    CT L = (h * (nc + nxp) * (Av[ic + 1] - ac) - h * (nc + nxm) * (ac - Av[ic - 1])) * ix2 +
+           (h * (nc + nyp) * (Av[ic + SX] - ac) - h * (nc + nym) * (ac - Av[ic - SX])) * iy2;
+    if constexpr (Z) L = L + (h * (nc + nzp) * (Ap[v * SPT + ic] - ac) - h * (nc + nzm) * (ac - am[v])) * iz2;
+    gout[v] = gout[v] + CT(nus[v == 0 ? 0 : (v == 4 ? 2 : 1)]) * L;
+  }
+}
+
+// Epilogue of one cell (each optional operand tested once): see the file comment.
+// Ac: the cell's adjoint input, component stride astr.
+template <class CT, class TIN, class TA, class TST>
+__device__ __forceinline__ void adj_epilogue(const GridDesc& g, const AdjArgs<TIN, TA, TST>& a, int b, int k, int gx,
+                                             int gy, size_t pbase, size_t fc, int cp, long long n5, const CT gin[5],
+                                             const CT lfv[5], const CT gout[5], const CT* Ac, int astr) {
+  CT gs[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) gs[v] = gin[v] + gout[v];
+  if (a.Gout) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) NS_ST(g, a.Gout, pbase + v * fc, cp, n5, gs[v]);
+  }
+  if (a.lam_out) {
+    double lv[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) lv[v] = widen(gs[v]);
+    if (a.lam_in) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) lv[v] = NS_LD(g, a.lam_in, pbase + v * fc, cp, n5) + lv[v];
+    }
+    if (a.obj_ndsc && (gx == a.obj_iL || gx == a.obj_iR)) {
+      // the objective source of this step on the plane's two columns, added after
+      // the stage products (the order of the separate scatter it replaces)
+      const int nf = g.ny * g.nz;
+      const double* Af = a.obj_aface + ((size_t)b * nf + (size_t)k * g.ny + gy) * 5;
+      const double NoD = a.obj_ndsc[2 * b], sc = a.obj_ndsc[2 * b + 1];
+      const int reps = (gx == a.obj_iL ? 1 : 0) + (gx == a.obj_iR ? 1 : 0);
+      for (int q = 0; q < reps; ++q) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) lv[v] += sc * (Af[v] - (v == 0 ? NoD : 0.0));
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < 5; ++v) NS_ST(g, a.lam_out, pbase + v * fc, cp, n5, lv[v]);
+    if (a.lam_out_mirror) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) NS_ST(g, a.lam_out_mirror, pbase + v * fc, cp, n5, cvt<TST>(lv[v]));
+    }
+  }
+  if (a.Anext) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v)
+      NS_ST(g, a.Anext, pbase + v * fc, cp, n5, CT(a.cl) * lfv[v] + CT(a.cg) * gout[v] + CT(a.cs) * gs[v]);
+  }
+  if (a.SBout || a.sbar) {
+    CT ss[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) ss[v] = Ac[v * astr];
+    if (a.SBin) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) ss[v] = NS_LD(g, a.SBin, pbase + v * fc, cp, n5) + ss[v];
+    }
+    if (a.SBout) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) NS_ST(g, a.SBout, pbase + v * fc, cp, n5, ss[v]);
+    }
+    if (a.sbar) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v)
+        NS_ST(g, a.sbar, pbase + v * fc, cp, n5, NS_LD(g, a.sbar, pbase + v * fc, cp, n5) + widen(ss[v]));
+    }
+  }
+}
 
 // values per face packet: 7 (viscous and face velocity), plus 10 with Roe dissipation
 template <bool ROE> constexpr int npk() { return ROE ? 17 : 7; }
@@ -606,16 +773,7 @@ __global__ void __launch_bounds__(NT, AdjMinBlocks<CT, ROE>::value) k_adj_stage(
         qb[2] = qb[2] + m23 * (own_m[2] - own_p[2]) * c.i4dx[2];
       }
       // ---- convective part and pull-back to conservative variables
-      const CT rho = Q0[ic];
-      const CT u[3] = {Q0[SP + ic], Q0[2 * SP + ic], Q0[3 * SP + ic]};
-      const CT e = Q0[4 * SP + ic];
-      const CT ir_ = CT(1) / rho;
-      const CT Esp = e + h * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);   // rho E / rho
-      const CT p = c.gm1 * rho * e;
-      const CT rE = rho * Esp;
-      CT rb = CT(0), mb[3] = {CT(0), CT(0), CT(0)}, Eb = CT(0), pb = CT(0);
-      CT ub[3] = {qb[0], qb[1], qb[2]};
-      CT eb = qb[3];
+      Convective<CT, SP> cv(c, Q0, ic, qb);
       if constexpr (ROE) {
         // Roe dissipation: the right-cell part of the lower faces and the left-cell part
         // of the upper faces, as adjoints of (rho, u, e)
@@ -627,137 +785,29 @@ __global__ void __launch_bounds__(NT, AdjMinBlocks<CT, ROE>::value) k_adj_stage(
           rs[v] = sFX[(12 + v) * TY * (TX + 1) + fl] + sFX[(7 + v) * TY * (TX + 1) + fl + 1] +
                   sFY[(12 + v) * (TY + 1) * TX + yl] + sFY[(7 + v) * (TY + 1) * TX + yl + TX] +
                   zlo[12 + v] + zhi[7 + v];
-        rb = rs[0];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) ub[j] = ub[j] + rs[1 + j];
-        eb = eb + rs[4];
+        cv.add_roe(rs);
       }
-      const int nb_lo[3] = {ic - 1, ic - SX, ic};
-      const int nb_hi[3] = {ic + 1, ic + SX, ic};
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const CT* Ahi = d == 2 ? Ap : A0;
+      {
         CT F[5];
 #pragma unroll
-        for (int v = 0; v < 5; ++v)
-          F[v] = (Ahi[v * SP + nb_hi[d]] - (d == 2 ? am[v] : A0[v * SP + nb_lo[d]])) * c.hidx[d];
-        const CT md = rho * u[d];
-        mb[d] = mb[d] + F[0] + F[1] * u[0] + F[2] * u[1] + F[3] * u[2];
+        for (int v = 0; v < 5; ++v) F[v] = (A0[v * SP + ic + 1] - A0[v * SP + ic - 1]) * c.hidx[0];
+        cv.template direction<0>(F);
 #pragma unroll
-        for (int j = 0; j < 3; ++j) ub[j] = ub[j] + F[1 + j] * md;
-        pb = pb + F[1 + d] + F[4] * u[d];
-        Eb = Eb + F[4] * u[d];
-        ub[d] = ub[d] + F[4] * (rE + p);
-      }
-      rb = rb + c.gm1 * e * pb;
-      eb = eb + c.gm1 * rho * pb;
-      Eb = Eb + eb * ir_;
-      rb = rb - eb * Esp * ir_;
+        for (int v = 0; v < 5; ++v) F[v] = (A0[v * SP + ic + SX] - A0[v * SP + ic - SX]) * c.hidx[1];
+        cv.template direction<1>(F);
 #pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        ub[j] = ub[j] - eb * u[j];
-        mb[j] = mb[j] + ub[j] * ir_;
-        rb = rb - ub[j] * u[j] * ir_;
+        for (int v = 0; v < 5; ++v) F[v] = (Ap[v * SP + ic] - am[v]) * c.hidx[2];
+        cv.template direction<2>(F);
       }
-      CT gout[5] = {rb, mb[0], mb[1], mb[2], Eb};
-      // ---- added adjoint viscosity L_nu a, times the factor of the component's state
-      // variable (rho, rho u, rho E)
+      CT gout[5];
+      cv.pull_back(c, gout);
+      // ---- added adjoint viscosity
       if (with_nu) {
         const CT* N0 = sN + s0 * SP;
-        const CT nc = N0[ic], nxm = N0[ic - 1], nxp = N0[ic + 1], nym = N0[ic - SX], nyp = N0[ic + SX],
-                 nzp = sN[sp * SP + ic];
-        const CT ix2 = c.idx[0] * c.idx[0], iy2 = c.idx[1] * c.idx[1], iz2 = c.idx[2] * c.idx[2];
-        int v0 = 0;
-        if constexpr (std::is_same<CT, float>::value) {
-          // components (0, 1) and (2, 3) side by side in paired FP32 instructions
-          const float2 fxp = f2(h * (nc + nxp), h * (nc + nxp)), fxm = f2(-h * (nc + nxm), -h * (nc + nxm));
-          const float2 fyp = f2(h * (nc + nyp), h * (nc + nyp)), fym = f2(-h * (nc + nym), -h * (nc + nym));
-          const float2 fzp = f2(h * (nc + nzp), h * (nc + nzp)), fzm = f2(-h * (nc + nzm), -h * (nc + nzm));
-#pragma unroll
-          for (int v = 0; v < 4; v += 2) {
-            const float* Av = A0 + v * SP;
-            const float* Aw = Av + SP;
-            const float2 ac = f2(Av[ic], Aw[ic]);
-            const float2 tx = __ffma2_rn(fxp, sub2(f2(Av[ic + 1], Aw[ic + 1]), ac),
-                                         __fmul2_rn(fxm, sub2(ac, f2(Av[ic - 1], Aw[ic - 1]))));
-            const float2 ty = __ffma2_rn(fyp, sub2(f2(Av[ic + SX], Aw[ic + SX]), ac),
-                                         __fmul2_rn(fym, sub2(ac, f2(Av[ic - SX], Aw[ic - SX]))));
-            const float2 tz = __ffma2_rn(fzp, sub2(f2(Ap[v * SP + ic], Ap[(v + 1) * SP + ic]), ac),
-                                         __fmul2_rn(fzm, sub2(ac, f2(am[v], am[v + 1]))));
-            const float2 L = __ffma2_rn(tz, f2(iz2, iz2), __ffma2_rn(ty, f2(iy2, iy2), __fmul2_rn(tx, f2(ix2, ix2))));
-            const float2 gv = __ffma2_rn(f2(float(a.nus[v == 0 ? 0 : 1]), float(a.nus[1])), L, f2(gout[v], gout[v + 1]));
-            gout[v] = gv.x;
-            gout[v + 1] = gv.y;
-          }
-          v0 = 4;
-        }
-#pragma unroll
-        for (int v = v0; v < 5; ++v) {
-          const CT* Av = A0 + v * SP;
-          const CT ac = Av[ic];
-          CT L = (h * (nc + nxp) * (Av[ic + 1] - ac) - h * (nc + nxm) * (ac - Av[ic - 1])) * ix2 +
-                 (h * (nc + nyp) * (Av[ic + SX] - ac) - h * (nc + nym) * (ac - Av[ic - SX])) * iy2 +
-                 (h * (nc + nzp) * (Ap[v * SP + ic] - ac) - h * (nc + nzm) * (ac - am[v])) * iz2;
-          gout[v] = gout[v] + CT(a.nus[v == 0 ? 0 : (v == 4 ? 2 : 1)]) * L;
-        }
+        add_viscosity<SP, true>(c, a.nus, A0, Ap, am, ic, N0[ic], N0[ic - 1], N0[ic + 1], N0[ic - SX], N0[ic + SX],
+                                nzm, sN[sp * SP + ic], gout);
       }
-      // ---- epilogue (each optional operand tested once per plane)
-      CT gs[5];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) gs[v] = gin[v] + gout[v];
-      if (a.Gout) {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) NS_ST(g, a.Gout, pbase + v * fc, cp, n5, gs[v]);
-      }
-      if (a.lam_out) {
-        double lv[5];
-#pragma unroll
-        for (int v = 0; v < 5; ++v) lv[v] = widen(gs[v]);
-        if (a.lam_in) {
-#pragma unroll
-          for (int v = 0; v < 5; ++v) lv[v] = NS_LD(g, a.lam_in, pbase + v * fc, cp, n5) + lv[v];
-        }
-        if (a.obj_ndsc && (gx == a.obj_iL || gx == a.obj_iR)) {
-          // the objective source of this step on the plane's two columns, added after
-          // the stage products (the order of the separate scatter it replaces)
-          const int nf = g.ny * g.nz;
-          const double* Af = a.obj_aface + ((size_t)b * nf + (size_t)k * g.ny + gy) * 5;
-          const double NoD = a.obj_ndsc[2 * b], sc = a.obj_ndsc[2 * b + 1];
-          const int reps = (gx == a.obj_iL ? 1 : 0) + (gx == a.obj_iR ? 1 : 0);
-          for (int q = 0; q < reps; ++q) {
-#pragma unroll
-            for (int v = 0; v < 5; ++v) lv[v] += sc * (Af[v] - (v == 0 ? NoD : 0.0));
-          }
-        }
-#pragma unroll
-        for (int v = 0; v < 5; ++v) NS_ST(g, a.lam_out, pbase + v * fc, cp, n5, lv[v]);
-        if (a.lam_out_mirror) {
-#pragma unroll
-          for (int v = 0; v < 5; ++v) NS_ST(g, a.lam_out_mirror, pbase + v * fc, cp, n5, cvt<TST>(lv[v]));
-        }
-      }
-      if (a.Anext) {
-#pragma unroll
-        for (int v = 0; v < 5; ++v)
-          NS_ST(g, a.Anext, pbase + v * fc, cp, n5, CT(a.cl) * lfv[v] + CT(a.cg) * gout[v] + CT(a.cs) * gs[v]);
-      }
-      if (a.SBout || a.sbar) {
-        CT ss[5];
-#pragma unroll
-        for (int v = 0; v < 5; ++v) ss[v] = A0[v * SP + ic];
-        if (a.SBin) {
-#pragma unroll
-          for (int v = 0; v < 5; ++v) ss[v] = NS_LD(g, a.SBin, pbase + v * fc, cp, n5) + ss[v];
-        }
-        if (a.SBout) {
-#pragma unroll
-          for (int v = 0; v < 5; ++v) NS_ST(g, a.SBout, pbase + v * fc, cp, n5, ss[v]);
-        }
-        if (a.sbar) {
-#pragma unroll
-          for (int v = 0; v < 5; ++v) NS_ST(g, a.sbar, pbase + v * fc, cp, n5, NS_LD(g, a.sbar, pbase + v * fc, cp, n5) + widen(ss[v]));
-        }
-      }
+      adj_epilogue(g, a, b, k, gx, gy, pbase, fc, cp, n5, gin, lfv, gout, A0 + ic, SP);
     }
 #pragma unroll
     for (int v = 0; v < NPK; ++v) zlo[v] = zhi[v];
@@ -770,6 +820,195 @@ __global__ void __launch_bounds__(NT, AdjMinBlocks<CT, ROE>::value) k_adj_stage(
   }
 }
 
+// ---------------------------------------------------------------------------------
+// 2D boxes (nz = 1).  Every z-difference of the product above is a difference of a plane
+// with itself, so the z-faces, the neighbouring planes and the march drop out and the
+// remaining operations give the same bits.  A CTA takes one tile of TX x TYF cells and
+// spreads the pieces of the product over its warps: the face s-vectors over all threads,
+// then one row of face packets per warp, then one (row, component) of the viscous
+// assembly per warp, then one row of cells per warp for the convective part and the
+// epilogue.  A 2D box has a few thousand to some ten thousand cells, so what counts is
+// the length of the dependent chain and the number of SMs at work, above all in FP64,
+// where one warp alone keeps its scheduler's FP64 unit busy.  One adjoint step (three
+// recomputed and four transposed stages), marching kernels before, these now: 64x64 FP64
+// 337 and 65 us, FP32 48 and 26 us; 400x400 FP64 1640 and 733 us, FP32 126 and 73 us.
+// ---------------------------------------------------------------------------------
+template <int TYF>
+struct FlatTile {
+  static constexpr int NW = 2 * TYF + 2;   // warps: TYF rows of x-faces, TYF + 1 of y-faces, the last x-faces
+  static constexpr int NT = 32 * NW;
+  static constexpr int SY = TYF + 2;
+  static constexpr int SP = SX * SY;
+  static constexpr int NX = SY * (SX - 1);        // x-faces with an s-vector
+  static constexpr int NF = NX + (SY - 1) * SX;   // and the y-faces
+};
+
+template <class CT, bool ROE, int TYF>
+constexpr size_t flat_smem_bytes() {
+  using T = FlatTile<TYF>;
+  return sizeof(CT) * (11 * T::SP + 4 * T::NF + npk<ROE>() * (TYF * (TX + 1) + (TYF + 1) * TX) + 4 * TYF * TX);
+}
+
+template <class CT, class TIN, class TA, class TST, bool ROE, int TYF>
+__global__ void __launch_bounds__(FlatTile<TYF>::NT) k_adj_flat(GridDesc g, Coef<CT> c, AdjArgs<TIN, TA, TST> a) {
+  using T = FlatTile<TYF>;
+  constexpr int SPT = T::SP, NFT = T::NF;
+  constexpr int NPK = npk<ROE>();
+  pdl_enter();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  CT* Q = reinterpret_cast<CT*>(smem_raw);   // [5][SP] primal primitives
+  CT* A = Q + 5 * SPT;                        // [5][SP] adjoint input a
+  CT* N = A + 5 * SPT;                        // [SP] added viscosity nu (when given)
+  CT* F = N + SPT;                            // [4][NF] face s-vectors, Fb[4]
+  CT* sFX = F + 4 * NFT;                      // [NPK][TYF][TX+1]
+  CT* sFY = sFX + NPK * TYF * (TX + 1);       // [NPK][TYF+1][TX]
+  CT* sQB = sFY + NPK * (TYF + 1) * TX;       // [4][TYF][TX] viscous adjoints of (u1, u2, u3, e)
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int ncx = (g.nx + TX - 1) / TX, ncy = (g.ny + TYF - 1) / TYF;
+  const int bx = blockIdx.x % ncx, r0 = blockIdx.x / ncx;
+  const int x0 = bx * TX, y0 = (r0 % ncy) * TYF, b = r0 / ncy;
+  const size_t box = (size_t)b * 5 * g.cells, fc = (size_t)g.cells;
+  const bool with_nu = a.nu != nullptr || a.nud != nullptr;
+  const long long n1 = g.cells * g.batch, n5 = 5 * n1;   // field extents (debug bounds checks)
+  (void)n1;
+  (void)n5;
+  const CT ca = CT(a.ca);
+  for (int t = tid; t < SPT; t += T::NT) {
+    const int ly = t / SX, lx = t - ly * SX;
+    const int o = wrap(y0 + ly - 1, g.ny) * g.nx + wrap(x0 + lx - 1, g.nx);
+    CT q[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      q[v] = cvt<CT>(NS_LD(g, a.W, box + v * fc, o, n5));
+      A[v * SPT + t] = ca * cvt<CT>(NS_LD(g, a.A, box + v * fc, o, n5));
+    }
+    if (a.nu) N[t] = CT(NS_LD(g, a.nu, (size_t)b * fc, o, n1));
+    else if (a.nud) N[t] = cvt<CT>(NS_LD(g, a.nud, (size_t)b * fc, o, n1));
+    const CT ir = CT(1) / q[0];
+    const CT u0 = q[1] * ir, u1 = q[2] * ir, u2 = q[3] * ir;
+    Q[t] = q[0];
+    Q[SPT + t] = u0;
+    Q[2 * SPT + t] = u1;
+    Q[3 * SPT + t] = u2;
+    Q[4 * SPT + t] = q[4] * ir - CT(0.5) * (u0 * u0 + u1 * u1 + u2 * u2);
+  }
+  __syncthreads();
+  for (int t = tid; t < NFT; t += T::NT) {
+    CT sv[3], fb4;
+    if (t < T::NX) {
+      const int row = t / (SX - 1);
+      const int iL = row * SX + (t - row * (SX - 1));
+      face_s<0, SPT>(c, Q, A, iL, Q, A, iL + 1, sv, fb4);
+    } else {
+      const int iL = t - T::NX;
+      face_s<1, SPT>(c, Q, A, iL, Q, A, iL + SX, sv, fb4);
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) F[j * NFT + t] = sv[j];
+    F[3 * NFT + t] = fb4;
+  }
+  __syncthreads();
+  auto xF = [&](int j, int row, int fx) { return F[j * NFT + row * (SX - 1) + fx]; };
+  auto yF = [&](int j, int fy, int col) { return F[j * NFT + T::NX + fy * SX + col]; };
+  const CT* u0 = Q + SPT;
+  const CT* v0 = Q + 2 * SPT;
+  if (wid < TYF || wid == T::NW - 1) {
+    // x-faces of row wid, or the rows' last ones
+    const int row = (wid < TYF ? wid : lane) + 1, fx = wid < TYF ? lane : TX;
+    if (row <= TYF) {
+      const int iL = row * SX + fx, iR = iL + 1;
+      CT gy[3] = {CT(0), CT(0), CT(0)}, gz[3] = {CT(0), CT(0), CT(0)}, pk[NPK];
+      diff4_pair(u0[iL + SX], u0[iL - SX], u0[iR + SX], u0[iR - SX], c.i4dx[1], v0[iL + SX], v0[iL - SX],
+                 v0[iR + SX], v0[iR - SX], c.i4dx[1], gy[0], gy[1]);
+      const CT sv[3] = {xF(0, row, fx), xF(1, row, fx), xF(2, row, fx)};
+      face_packet_s<0, SPT>(c, sv, xF(3, row, fx), Q, iL, Q, iR, gy, gz, pk);
+      if constexpr (ROE) roe_packet<0, SPT>(c, Q, A, iL, Q, A, iR, pk + 7);
+#pragma unroll
+      for (int v = 0; v < NPK; ++v) sFX[(v * TYF + row - 1) * (TX + 1) + fx] = pk[v];
+    }
+  } else {
+    const int fy = wid - TYF, iL = fy * SX + lane + 1, iR = iL + SX;
+    CT gz[3] = {CT(0), CT(0), CT(0)}, gx[3] = {CT(0), CT(0), CT(0)}, pk[NPK];
+    diff4_pair(v0[iL + 1], v0[iL - 1], v0[iR + 1], v0[iR - 1], c.i4dx[0], u0[iL + 1], u0[iL - 1], u0[iR + 1],
+               u0[iR - 1], c.i4dx[0], gx[1], gx[0]);
+    const CT sv[3] = {yF(0, fy, lane + 1), yF(1, fy, lane + 1), yF(2, fy, lane + 1)};
+    face_packet_s<1, SPT>(c, sv, yF(3, fy, lane + 1), Q, iL, Q, iR, gz, gx, pk);
+    if constexpr (ROE) roe_packet<1, SPT>(c, Q, A, iL, Q, A, iR, pk + 7);
+#pragma unroll
+    for (int v = 0; v < NPK; ++v) sFY[(v * (TYF + 1) + fy) * TX + lane] = pk[v];
+  }
+  __syncthreads();
+  // viscous part, component v of (u1, u2, u3, e) of row ty
+  for (int job = wid; job < 4 * TYF; job += T::NW) {
+    const int v = job & 3, ty = job >> 2, tx = lane;
+    const CT m = c.mu, m23 = CT(-2.0 / 3.0) * c.mu;
+    const CT* px = sFX + (v * TYF + ty) * (TX + 1) + tx;
+    const CT* py = sFY + (v * (TYF + 1) + ty) * TX + tx;
+    CT qb = (px[0] - px[1]) * c.idx[0] + (py[0] - py[TX]) * c.idx[1];
+    if (v < 3) {
+      const CT* ux = px + 4 * TYF * (TX + 1);
+      const CT* uy = py + 4 * (TYF + 1) * TX;
+      qb = qb + CT(0.5) * (ux[0] + ux[1] + uy[0] + uy[TX]);
+    }
+    // the tangential parts (see the marching kernel); T[z][*] and T[*][z] vanish
+    auto Sy = [&](int j, int col) { return yF(j, ty, col) + yF(j, ty + 1, col); };
+    auto Sx = [&](int j, int row) { return xF(j, row, tx) + xF(j, row, tx + 1); };
+    if (v == 0) {
+      qb = qb + m23 * (Sy(1, tx) - Sy(1, tx + 2)) * c.i4dx[0];
+      qb = qb + m * (Sx(1, ty) - Sx(1, ty + 2)) * c.i4dx[1];
+    } else if (v == 1) {
+      qb = qb + m * (Sy(0, tx) - Sy(0, tx + 2)) * c.i4dx[0];
+      qb = qb + m23 * (Sx(0, ty) - Sx(0, ty + 2)) * c.i4dx[1];
+    }
+    sQB[(v * TYF + ty) * TX + tx] = qb;
+  }
+  __syncthreads();
+  for (int ty = wid; ty < TYF; ty += T::NW) {
+    const int tx = lane, gx = x0 + tx, gy = y0 + ty;
+    if (gx >= g.nx || gy >= g.ny) continue;
+    const int ic = (ty + 1) * SX + tx + 1, cp = gy * g.nx + gx;
+    CT gin[5] = {CT(0), CT(0), CT(0), CT(0), CT(0)};
+    CT lfv[5] = {CT(0), CT(0), CT(0), CT(0), CT(0)};
+    if (a.Gin) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) gin[v] = NS_LD(g, a.Gin, box + v * fc, cp, n5);
+    }
+    if (a.Anext) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) lfv[v] = NS_LD(g, a.lamf, box + v * fc, cp, n5);
+    }
+    CT rs[5] = {CT(0), CT(0), CT(0), CT(0), CT(0)};
+    if constexpr (ROE) {
+      const int fl = ty * (TX + 1) + tx, yl = ty * TX + tx;
+#pragma unroll
+      for (int v = 0; v < 5; ++v)
+        rs[v] = sFX[(12 + v) * TYF * (TX + 1) + fl] + sFX[(7 + v) * TYF * (TX + 1) + fl + 1] +
+                sFY[(12 + v) * (TYF + 1) * TX + yl] + sFY[(7 + v) * (TYF + 1) * TX + yl + TX];
+    }
+    CT qb[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) qb[v] = sQB[(v * TYF + ty) * TX + tx];
+    Convective<CT, SPT> cv(c, Q, ic, qb);
+    if constexpr (ROE) cv.add_roe(rs);
+    {
+      CT D[5];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) D[v] = (A[v * SPT + ic + 1] - A[v * SPT + ic - 1]) * c.hidx[0];
+      cv.template direction<0>(D);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) D[v] = (A[v * SPT + ic + SX] - A[v * SPT + ic - SX]) * c.hidx[1];
+      cv.template direction<1>(D);
+    }
+    CT gout[5];
+    cv.pull_back(c, gout);
+    if (with_nu) {
+      const CT nc = N[ic], nxm = N[ic - 1], nxp = N[ic + 1], nym = N[ic - SX], nyp = N[ic + SX];
+      add_viscosity<SPT, false>(c, a.nus, A, A, static_cast<const CT*>(nullptr), ic, nc, nxm, nxp, nym, nyp, CT(0), CT(0), gout);
+    }
+    adj_epilogue(g, a, b, 0, gx, gy, box, fc, cp, n5, gin, lfv, gout, A + ic, SPT);
+  }
+}
+
 template <class CT, bool ROE>
 size_t adj_smem_bytes() {
   constexpr int NPK = npk<ROE>();
@@ -777,9 +1016,30 @@ size_t adj_smem_bytes() {
          (3 * 5 * SP * 2 + 2 * 4 * NF + 2 * 3 * SP + NPK * TY * (TX + 1) + NPK * (TY + 1) * TX + 3 * SP);
 }
 
+template <class CT, class TIN, class TA, class TST, bool ROE, int TYF>
+static cudaError_t launch_adj_flat(const GridDesc& g, const Coef<CT>& c, const AdjArgs<TIN, TA, TST>& a,
+                                   cudaStream_t st) {
+  constexpr size_t smem = flat_smem_bytes<CT, ROE, TYF>();
+  auto kern = k_adj_flat<CT, TIN, TA, TST, ROE, TYF>;
+  static FlatShape<TYF> shape;
+  int ctas = 0;
+  cudaError_t e = shape.get(kern, smem, g, ctas);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(kern, dim3(ctas), dim3(FlatTile<TYF>::NT), smem, st, g, c, a);
+  count_launch();
+  return e;
+}
+
 template <class CT, class TIN, class TA, class TST, bool ROE>
 static cudaError_t launch_adj_variant(const GridDesc& g, const Coef<CT>& c, const AdjArgs<TIN, TA, TST>& a,
                                      cudaStream_t st) {
+  // 2D boxes; the FP32 Roe product stays with the marching kernel, whose rounding of the
+  // dissipation's transpose the flat kernel does not reproduce
+  if constexpr (!(ROE && std::is_same<CT, float>::value)) {
+    if (g.nz == 1)
+      return flat_rows(g) == 1 ? launch_adj_flat<CT, TIN, TA, TST, ROE, 1>(g, c, a, st)
+                               : launch_adj_flat<CT, TIN, TA, TST, ROE, 4>(g, c, a, st);
+  }
   const size_t smem = adj_smem_bytes<CT, ROE>();
   auto kern = k_adj_stage<CT, TIN, TA, TST, ROE>;
   static MarchShape<TX, TY> shape;

@@ -96,6 +96,37 @@ struct MarchShape {
   }
 };
 
+// Launch shape of the 2D (nz = 1) stage kernels: one CTA per tile of TX x TYF cells; the
+// kernel's dynamic shared-memory limit is raised once per device.
+template <int TYF>
+struct FlatShape {
+  bool ready[16] = {false};
+  template <class K>
+  cudaError_t get(K kern, size_t smem, const GridDesc& g, int& ctas) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 16 || !ready[dev]) {
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+      if (dev >= 0 && dev < 16) ready[dev] = true;
+    }
+    const long long n = (long long)((g.nx + TX - 1) / TX) * ((g.ny + TYF - 1) / TYF) * g.batch;
+    if (n > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
+    ctas = (int)n;
+    return cudaSuccess;
+  }
+};
+
+// Rows per tile of the 2D kernels: single rows spread a small box over the most SMs and
+// keep the chain of a CTA shortest, but compute each y-face twice; four rows share them.
+// Single rows up to two CTAs per SM: one FP64 step at 64x64 (128 single-row tiles) takes
+// 23 us with single rows and 42 us with four, at 128x128 (512 tiles) 61 and 42 us.
+inline int flat_rows(const GridDesc& g) {
+  const long long rows = (long long)((g.nx + TX - 1) / TX) * g.ny * g.batch;
+  return rows <= 2 * 152 ? 1 : 4;
+}
+
 template <class T>
 struct Coef {
   T gamma, gm1, mu, alpha;
