@@ -184,6 +184,8 @@ static int adjoint_step_t(ns_ctx* c, const Coef<CT>& cf, const CT* W1, const CT*
   prof_mark(c);
   for (int j = 0; j < sc.ns; ++j) {
     const bool last = j == sc.ns - 1;
+    // only the last stage adds the objective source formed on the side stream
+    if (last && obj && ns_i_objective_join(c) != NS_OK) return NS_ERR_CUDA;
     CT* Aout = last ? nullptr : (j % 2 == 0 ? Aa : Ab);
     ns::AdjArgs<CT, CT, CT> a{};
     a.W = last ? W1 : Wst[sc.ns - 2 - j];

@@ -507,7 +507,8 @@ int adjoint_at(ns_ctx* c, ns_sweep_state& S, int n, const double* w, const void*
   const float* nup = nullptr;
   const double* nudp = nullptr;
   // the objective of w^n (n >= 1): its plane sums on the side stream, concurrent with
-  // sigma_1, its source folded into the last transposed stage of this step
+  // sigma_1 and the first transposed stages; its source is folded into the step's last
+  // transposed stage, which waits for them
   ns_obj_src obj{};
   if (n >= 1 && (r = ns_i_objective_sum_forked(c, w, wN, S.jtmp, &obj))) return r;
   if (need_sigma && S.f64nu) {
@@ -531,7 +532,6 @@ int adjoint_at(ns_ctx* c, ns_sweep_state& S, int n, const double* w, const void*
       nup = S.nu;
     }
   }
-  if (n >= 1 && (r = ns_i_objective_join(c))) return r;
   if ((r = ns_i_adjoint(c, w, mirror, kept3, S.s, lam_cur,
                         S.lamf_valid ? S.lamf_cur : nullptr, nup, lam_nxt, S.lamf_nxt, sbar, nudp,
                         n >= 1 ? &obj : nullptr)))
