@@ -226,7 +226,9 @@ int ns_max_wave_speed(ns_ctx* ctx, const double* w, double* out);
  * segments recomputed during the backward sweep).  The host runtime plans which
  * primal states to keep (ns_plan) and executes the plan on the context's stream
  * (ns_adjoint_run).  Schedules:
- *   NS_CKPT_ALL     keep every state (no recomputation)
+ *   NS_CKPT_ALL     keep every state, and on a periodic box every step's stage states when
+ *                   they take at most 16 GiB (no recomputation; without them, and after
+ *                   ns_set_pipeline(ctx, 0), each adjoint step recomputes its stages)
  *   NS_CKPT_STRIDE  keep every param-th state; replay one segment at a time and keep
  *                   all its states during its reversal.  The last segment is not
  *                   replayed: the forward pass keeps its states, so a sweep advances
@@ -334,7 +336,8 @@ typedef struct {
 
 /* Device bytes the caller must provide as the arena of ns_adjoint_run (state slots,
  * two working states, one adjoint field, sigma_1 and nu fields, scalars; for a stride
- * plan one segment's kept stage states and mirrors, and when the sweep is pipelined a
+ * plan one segment's kept stage states and mirrors, for a store-all plan every step's while
+ * they take at most 16 GiB, and when the sweep is pipelined a
  * second set of them with param - 1 segment states per set, see ns_set_pipeline). */
 size_t ns_run_arena_bytes(const ns_ctx* ctx, const ns_run_opts* o);
 
@@ -373,8 +376,9 @@ int ns_backward_run(ns_ctx* ctx, double* lam0, double* sbar, double* energy, dou
  * forward's trajectory.  The paper has no counterpart. */
 long long ns_sweep_generation(const ns_ctx* ctx);
 
-/* Pipelined stride sweeps on this context (NS_CKPT_STRIDE above): on = 1 (the default
- * unless the environment sets NS_PIPELINE=0) or 0.  The pipelined arena holds a second
+/* Pipelined stride sweeps and kept stages of store-all sweeps on this context
+ * (NS_CKPT_STRIDE, NS_CKPT_ALL above): on = 1 (the default unless the environment sets
+ * NS_PIPELINE=0) or 0, the smallest device footprint.  The pipelined arena holds a second
  * set of param - 1 segment states and of kept stages (ns_run_arena_bytes follows the
  * setting); its replays run on a context the library creates on first use with this
  * context's parameters, which reports into this context's error word.  NS_ERR_ARG for a

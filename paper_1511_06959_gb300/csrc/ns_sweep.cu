@@ -326,7 +326,8 @@ bool file_io(int fd, void* buf, size_t n, long long off, bool write) {
 // Arena regions.  mir: two stage-type fields holding float mirrors of consecutive
 // states of an ADVANCE run (mixed precision).  lmir: two float mirrors of the adjoint,
 // written by the last adjoint stage and kept in step by the objective source, so that
-// the next adjoint step needs no conversion (mixed precision).  keep: for stride schedules, one entry of
+// the next adjoint step needs no conversion (mixed precision).  keep: for stride schedules (and
+// store-all ones with room for every step), one entry of
 // four stage-type fields per step of the segment being reversed (the mirror of w^n and
 // the stage states W2..W4 computed when the segment was replayed), so that the adjoint
 // of a replayed step neither recomputes its stages nor converts its state.
@@ -357,8 +358,23 @@ bool pipelined(const ns_ctx* c, int nsteps, int schedule, int param, bool verify
          param >= 2 && nsteps - 1 >= param;
 }
 
+// A store-all sweep also keeps every step's stage states from the forward pass, as the
+// stride plans do for the segment being reversed, so that its adjoint steps recompute
+// nothing: three of the eleven stage launches per RK4 step (a batch of eight 96x48x48
+// boxes, 20 steps with gradients: 24.5 ms without, 19.1 ms with).  It does so while they
+// take at most KEEP_ALL_MAX bytes (about a sixteenth of the device's 280 GB) and unless
+// the caller asked for the smallest footprint (ns_set_pipeline(ctx, 0), NS_PIPELINE=0).
+constexpr size_t KEEP_ALL_MAX = (size_t)16 << 30;
+
+bool keeps_all_stages(const ns_ctx* c, int nsteps, int schedule) {
+  const bool on = c->pipeline < 0 ? pipeline_enabled() : c->pipeline != 0;
+  return on && schedule == NS_CKPT_ALL && !c->bounded() &&
+         (size_t)nsteps <= KEEP_ALL_MAX / 4 / align256(ns_i_stage_bytes(c));
+}
+
+// keep_all: the number of steps whose stages a store-all sweep keeps (0: none)
 Layout layout_for(const ns_ctx* c, int slots_used, bool closure, int schedule, int param, int host_slots = 0,
-                  bool verify = false, bool pipe = false) {
+                  bool verify = false, bool pipe = false, int keep_all = 0) {
   // a bounded box forms its stage states inside its own step calls: nothing is kept
   if (c->bounded()) schedule = -1;
   Layout L;
@@ -377,7 +393,7 @@ Layout layout_for(const ns_ctx* c, int slots_used, bool closure, int schedule, i
   L.lmir = c->p.precision == NS_MIXED ? 2 * L.stage : 0;
   L.nkeep = (schedule == NS_CKPT_STRIDE || schedule == NS_CKPT_STRIDE_HOST || schedule == NS_CKPT_STRIDE_DISK)
                 ? param
-                : 0;
+                : keep_all;
   L.keep = (size_t)L.nkeep * 4 * L.stage;
   // snapshot checksums: one per device slot and per host slot, and one to verify into
   L.sums = verify ? align256(sizeof(unsigned long long) * (size_t)(slots_used + host_slots + 1)) : 0;
@@ -413,7 +429,8 @@ size_t ns_run_arena_bytes(const ns_ctx* c, const ns_run_opts* o) {
   Planner P;
   if (make_plan(o->nsteps, o->schedule, o->param, P)) return 0;
   return layout_for(c, P.maxlive, o->mlp != nullptr, o->schedule, o->param, P.maxhost, o->verify != 0,
-                    pipelined(c, o->nsteps, o->schedule, o->param, o->verify != 0))
+                    pipelined(c, o->nsteps, o->schedule, o->param, o->verify != 0),
+                    keeps_all_stages(c, o->nsteps, o->schedule) ? o->nsteps : 0)
       .total;
 }
 
@@ -580,7 +597,8 @@ int run_actions(ns_ctx* c, ns_sweep_state& S, int stop_op, double*& lam_cur, dou
           if (out < 0) return NS_ERR_BUDGET;
           const int K = S.L.nkeep;
           // the stride plans replay every segment but the last, whose states they keep from
-          // the forward pass: its steps keep their stages there
+          // the forward pass: its steps keep their stages there (a store-all plan is one
+          // segment)
           const bool keep = K > 0 && !S.bounded && (S.in_backward || n >= ((N - 1) / K) * K);
           void* in_m = S.mixed && !S.bounded ? S.cur_mirror : nullptr;
           void* out_m = nullptr;
@@ -880,7 +898,7 @@ static int forward_run_impl(ns_ctx* c, const double* w0, const double* s, const 
   }
   S->pipe = pipelined(c, o->nsteps, o->schedule, o->param, o->verify != 0);
   S->L = layout_for(c, S->P.maxlive, o->mlp != nullptr, o->schedule, o->param, S->P.maxhost, o->verify != 0,
-                    S->pipe);
+                    S->pipe, keeps_all_stages(c, o->nsteps, o->schedule) ? o->nsteps : 0);
   if (arena_bytes < S->L.total) {
     delete S;
     return NS_ERR_BUDGET;
