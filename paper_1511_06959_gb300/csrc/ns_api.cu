@@ -661,11 +661,7 @@ int ns_growth_sigma1(ns_ctx* c, const double* w, float* sigma1, double* stats) {
     if (stats) return NS_ERR_ARG;
     return mixed(c) ? bounded_sigma1_t<float>(c, w, sigma1, nullptr) : bounded_sigma1_t<double>(c, w, sigma1, nullptr);
   }
-  if (mixed(c)) {
-    float* wf = buf<float>(c, WF);
-    if (ns::launch_to_float(w, wf, c->field, c->st) != cudaSuccess) return NS_ERR_CUDA;
-    return cuerr(ns::launch_sigma1<float>(c->g, c->cf, wf, sigma1, stats, c->scratch, c->ticket, c->st));
-  }
+  if (mixed(c)) return cuerr(ns::launch_sigma1<float>(c->g, c->cf, w, sigma1, stats, c->scratch, c->ticket, c->st));
   return cuerr(ns::launch_sigma1<double>(c->g, c->cd, w, sigma1, stats, c->scratch, c->ticket, c->st));
 }
 
@@ -937,13 +933,10 @@ int ns_i_sigma1(ns_ctx* c, const double* w, const void* w_mirror, float* sigma1,
   ns::NuRule rule{(float)lambda, (float)tau, (float)nu_limit(c), nu, c->err, 0.0, 0.0, 0.0, nullptr, c->nu_cap};
   const ns::NuRule* rp = nu ? &rule : nullptr;
   if (mixed(c)) {
-    const float* wf = (const float*)w_mirror;
-    if (!wf) {
-      float* t = buf<float>(c, WF);
-      if (ns::launch_to_float(w, t, c->field, c->st) != cudaSuccess) return NS_ERR_CUDA;
-      wf = t;
-    }
-    return cuerr(ns::launch_sigma1<float>(c->g, c->cf, wf, sigma1, stats, c->scratch, c->ticket, c->st, rp));
+    if (!w_mirror)
+      return cuerr(ns::launch_sigma1<float>(c->g, c->cf, w, sigma1, stats, c->scratch, c->ticket, c->st, rp));
+    return cuerr(ns::launch_sigma1<float>(c->g, c->cf, (const float*)w_mirror, sigma1, stats, c->scratch, c->ticket,
+                                          c->st, rp));
   }
   return cuerr(ns::launch_sigma1<double>(c->g, c->cd, w, sigma1, stats, c->scratch, c->ticket, c->st, rp));
 }

@@ -152,34 +152,38 @@ __device__ __forceinline__ int wrap(int i, int n) {
 //        (2^-126) flush to signed zero; overflow gives infinity; NaN stays NaN.
 //   f2d: exact for normal floats and zero; subnormal floats flush to signed zero.
 // ---------------------------------------------------------------------------------
+// Normal and zero values take a straight line of integer instructions (about a dozen; a
+// form that branched on each range took twice as many); infinities, NaN and overflow
+// branch off.
 __device__ __forceinline__ float d2f(double x) {
   const unsigned hi = (unsigned)__double2hiint(x);
   const unsigned lo = (unsigned)__double2loint(x);
   const unsigned sign = hi & 0x80000000u;
-  const int e = (int)((hi >> 20) & 0x7FFu);
-  const unsigned frac_hi = hi & 0xFFFFFu;            // top 20 fraction bits
-  if (e == 0x7FF) {                                   // inf / nan
-    const bool nan = (frac_hi | lo) != 0u;
-    return __uint_as_float(sign | 0x7F800000u | (nan ? 0x00400000u : 0u));
+  const int m = (int)(hi & 0x7FFFFFFFu) - (896 << 20);   // biased exponent of the result above 20 fraction bits
+  unsigned r = __funnelshift_l(lo, (unsigned)m, 3);       // the result's 31 bits before rounding
+  // up when the 29 dropped bits exceed one half, or equal it and the result is odd
+  r += ((lo & 0x1FFFFFFFu) + (r & 1u) + 0x0FFFFFFFu) >> 29;   // a carry may reach infinity
+  if (m < (1 << 20)) r = 0u;                                   // zero, subnormal, underflow
+  if (m >= (255 << 20)) {
+    const bool nan = (hi & 0x7FFFFFFFu) > 0x7FF00000u || ((hi & 0x7FFFFFFFu) == 0x7FF00000u && lo != 0u);
+    r = 0x7F800000u | (nan ? 0x00400000u : 0u);
   }
-  const int fe = e - 1023 + 127;
-  if (fe <= 0) return __uint_as_float(sign);          // zero, subnormal, underflow
-  if (fe >= 255) return __uint_as_float(sign | 0x7F800000u);
-  const unsigned fm = (frac_hi << 3) | (lo >> 29);    // 23 fraction bits
-  const unsigned rem = lo & 0x1FFFFFFFu;              // 29 dropped bits
-  unsigned r = sign | ((unsigned)fe << 23) | fm;
-  if (rem > 0x10000000u || (rem == 0x10000000u && (fm & 1u))) r += 1u;   // carry may reach inf
-  return __uint_as_float(r);
+  return __uint_as_float(sign | r);
 }
 
 __device__ __forceinline__ double f2d(float f) {
   const unsigned u = __float_as_uint(f);
-  const unsigned sign = u & 0x80000000u;
-  const unsigned e = (u >> 23) & 0xFFu;
-  const unsigned m = u & 0x7FFFFFu;
-  if (e == 0u) return __hiloint2double((int)sign, 0);
-  if (e == 0xFFu) return __hiloint2double((int)(sign | 0x7FF00000u | (m >> 3) | (m ? 0x80000u : 0u)), 0);
-  return __hiloint2double((int)(sign | ((e + 896u) << 20) | (m >> 3)), (int)(m << 29));
+  const unsigned sign = u & 0x80000000u, a = u & 0x7FFFFFFFu;
+  unsigned hi = (a >> 3) + (896u << 20), lo = u << 29;
+  if (a < 0x00800000u) {   // zero, subnormal
+    hi = 0u;
+    lo = 0u;
+  }
+  if (a >= 0x7F800000u) {   // infinity, NaN (kept, made quiet)
+    const unsigned m = u & 0x7FFFFFu;
+    hi = 0x7FF00000u | (m >> 3) | (m ? 0x80000u : 0u);
+  }
+  return __hiloint2double((int)(sign | hi), (int)lo);
 }
 
 // conversions used by the templated kernels: to the compute type / back to FP64
@@ -245,6 +249,21 @@ __device__ __forceinline__ void diff4_pair(CT a1, CT b1, CT c1, CT d1, CT s1, CT
     r1 = (a1 - b1 + c1 - d1) * s1;
     r2 = (a2 - b2 + c2 - d2) * s2;
   }
+}
+
+// (hi, lo) += (bhi, blo) for unevaluated float pairs hi + lo: Knuth's two-sum of the high
+// parts, the low parts added to its error, then a renormalising fast two-sum.  The pair
+// keeps the sum of float terms to about 2^-44 relative; the result does not depend on
+// the order of the two operands.
+// (The explicit roundings keep a product in an operand from being fused into the sums,
+// which would break the error-free transformation.)
+__device__ __forceinline__ void df_add(float& hi, float& lo, float bhi, float blo) {
+  const float s = __fadd_rn(hi, bhi);
+  const float bb = __fsub_rn(s, hi);
+  float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(bhi, bb));
+  e = __fadd_rn(e, __fadd_rn(lo, blo));
+  hi = __fadd_rn(s, e);
+  lo = __fsub_rn(e, __fsub_rn(hi, s));
 }
 
 // ---------------------------------------------------------------------------------

@@ -473,19 +473,6 @@ __device__ __forceinline__ void growth_matrix(const GridDesc& g, const Coef<CT>&
   M[4][4] -= gm1 / CT(2) * div;
 }
 
-// (hi, lo) += (bhi, blo) for unevaluated float pairs hi + lo: Knuth's two-sum of the high
-// parts, the low parts added to its error, then a renormalising fast two-sum.  The pair
-// keeps the sum of float terms to about 2^-44 relative; the result does not depend on
-// the order of the two operands.
-__device__ __forceinline__ void df_add(float& hi, float& lo, float bhi, float blo) {
-  const float s = hi + bhi;
-  const float bb = s - hi;
-  float e = (hi - (s - bb)) + (bhi - bb);
-  e = e + (lo + blo);
-  hi = s + e;
-  lo = e - (hi - s);
-}
-
 // sigma_1 by plane marching.  A CTA owns a TX x SG_TY tile of columns and a range of
 // planes (march_range, as the stencil kernels); the primitives (rho, u1, u2, u3, p, a, b)
 // of three consecutive planes of the tile and its one-cell halo sit in a shared-memory
@@ -509,9 +496,11 @@ size_t sigma1_march_ctas_bound(const GridDesc& g) {
   return (size_t)(cols > 2048 ? cols : 2048);
 }
 
-template <class CT>
+// TIN: the state's type; a mixed-precision context's FP64 state is rounded as it is loaded
+// (the bits of a converted copy, whose pass over memory cost 8 us of 128x64x64 cells).
+template <class CT, class TIN>
 __global__ void __launch_bounds__(sgk::NT, sizeof(CT) == 4 ? 4 : 1) k_sigma1(GridDesc g, Coef<CT> c,
-                                                                          const CT* __restrict__ w,
+                                                                          const TIN* __restrict__ w,
                                                                           float* __restrict__ sig, double* partial,
                                                                           double* stats, unsigned* ticket,
                                                                           NuRule rule, double* __restrict__ sigd) {
@@ -544,7 +533,7 @@ __global__ void __launch_bounds__(sgk::NT, sizeof(CT) == 4 ? 4 : 1) k_sigma1(Gri
     for (int it = 0; it < 2; ++it)
       if (tid + it * NT < SP) {
 #pragma unroll
-        for (int v = 0; v < 5; ++v) q[it][v] = w[pb + v * (size_t)g.cells + ho[it]];
+        for (int v = 0; v < 5; ++v) q[it][v] = cvt<CT>(w[pb + v * (size_t)g.cells + ho[it]]);
       }
   };
   auto store = [&](const CT (&q)[2][5], int slot) {
@@ -747,6 +736,7 @@ __device__ __forceinline__ void vhat_cell(const CT* __restrict__ w, const double
 template <class CT>
 __global__ void __launch_bounds__(RB) k_label(GridDesc g, Coef<CT> c, const CT* __restrict__ w,
                                               const double* __restrict__ lam, float* __restrict__ acc) {
+  pdl_enter();
   const long long i = (long long)blockIdx.x * RB + threadIdx.x;
   if (i >= g.cells * g.batch) return;
   const int b = (int)(i / g.cells);
@@ -791,6 +781,7 @@ __global__ void __launch_bounds__(RB) k_label(GridDesc g, Coef<CT> c, const CT* 
 // ---------------------------------------------------------------------------------
 __global__ void k_nu_rule(long long n, const float* __restrict__ s1, float lam, float tau,
                           float limit_nu, float* __restrict__ nu, unsigned* err, bool cap) {
+  pdl_enter();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float s = s1[i];
@@ -800,6 +791,7 @@ __global__ void k_nu_rule(long long n, const float* __restrict__ s1, float lam, 
 // the same rule in FP64 (FP64 contexts)
 __global__ void k_nu_rule_f64(long long n, const double* __restrict__ s1, double lam, double tau,
                               double limit_nu, double* __restrict__ nu, unsigned* err, bool cap) {
+  pdl_enter();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double s = s1[i];
@@ -809,6 +801,7 @@ __global__ void k_nu_rule_f64(long long n, const double* __restrict__ s1, double
 __global__ void k_visc_apply(GridDesc g, double ix2, double iy2, double iz2, double f_rho, double f_mom,
                              double f_en, const float* __restrict__ nu, const double* __restrict__ a,
                              double* __restrict__ out) {
+  pdl_enter();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long tot = g.cells * g.batch;
   if (i >= tot) return;
@@ -917,6 +910,7 @@ __global__ void __launch_bounds__(RB, sizeof(T) == 4 ? 8 : 1) k_energy(GridDesc 
 
 __global__ void __launch_bounds__(RB) k_sum_partials(int nblk, double scale, const double* partial,
                                                      double* out, unsigned* err) {
+  pdl_enter();
   __shared__ double sh[RB];
   const int b = blockIdx.x;
   double s = 0.0;
@@ -934,6 +928,7 @@ __global__ void __launch_bounds__(RB) k_sum_partials(int nblk, double scale, con
 // ---------------------------------------------------------------------------------
 __global__ void __launch_bounds__(RB) k_dot(const double* __restrict__ a, const double* __restrict__ phi,
                                             size_t n, double* partial) {
+  pdl_enter();
   __shared__ double sh[RB];
   const int m = blockIdx.y;
   const double* pm = phi + (size_t)m * n;
@@ -945,6 +940,7 @@ __global__ void __launch_bounds__(RB) k_dot(const double* __restrict__ a, const 
 
 __global__ void k_combine(const double* __restrict__ theta, const double* __restrict__ phi, int nphi,
                           size_t n, double* __restrict__ s) {
+  pdl_enter();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double acc = 0.0;
@@ -954,6 +950,7 @@ __global__ void k_combine(const double* __restrict__ theta, const double* __rest
 
 __global__ void __launch_bounds__(RB) k_max_wave(GridDesc g, double gamma, const double* __restrict__ w,
                                                  double* partial) {
+  pdl_enter();
   __shared__ double sh[RB];
   double mx = 0.0;
   const long long tot = g.cells * g.batch;
@@ -972,6 +969,7 @@ __global__ void __launch_bounds__(RB) k_max_wave(GridDesc g, double gamma, const
 }
 
 __global__ void __launch_bounds__(RB) k_max_partials(int nblk, const double* partial, double* out) {
+  pdl_enter();
   __shared__ double sh[RB];
   double m = 0.0;
   for (int i = threadIdx.x; i < nblk; i += RB) m = fmax(m, partial[i]);
@@ -980,6 +978,7 @@ __global__ void __launch_bounds__(RB) k_max_partials(int nblk, const double* par
 }
 
 __global__ void k_scale_boxes(GridDesc g, const double* __restrict__ seed, double* __restrict__ field) {
+  pdl_enter();
   const long long tot = g.cells * 5 * g.batch;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < tot) field[i] *= seed[i / (g.cells * 5)];
@@ -987,6 +986,7 @@ __global__ void k_scale_boxes(GridDesc g, const double* __restrict__ seed, doubl
 
 __global__ void __launch_bounds__(RB) k_dot_boxes(GridDesc g, const double* __restrict__ field, int comp,
                                                   const double* __restrict__ phi, double* partial) {
+  pdl_enter();
   __shared__ double sh[RB];
   const int m = blockIdx.y;
   const double* pm = phi + (size_t)m * g.cells;
@@ -1003,6 +1003,7 @@ __global__ void __launch_bounds__(RB) k_dot_boxes(GridDesc g, const double* __re
 // relative change of a sensitivity field: sum (b - a)^2 and sum b^2 over n elements
 __global__ void __launch_bounds__(RB) k_diff_norms(const double* __restrict__ a, const double* __restrict__ b,
                                                    size_t n, double* partial) {
+  pdl_enter();
   __shared__ double sh[RB];
   double d2 = 0.0, b2 = 0.0;
   for (size_t i = (size_t)blockIdx.x * RB + threadIdx.x; i < n; i += (size_t)gridDim.x * RB) {
@@ -1019,6 +1020,7 @@ __global__ void __launch_bounds__(RB) k_diff_norms(const double* __restrict__ a,
 }
 
 __global__ void k_to_float(const double* __restrict__ in, float* __restrict__ out, size_t n) {
+  pdl_enter();
   const size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 2;
   if (i + 1 < n) {
     const double2 v = *reinterpret_cast<const double2*>(in + i);
@@ -1101,35 +1103,36 @@ cudaError_t launch_objective_sum(const GridDesc& g, double gamma, int plane_i, d
   return e;
 }
 
-template <class CT>
-cudaError_t launch_sigma1(const GridDesc& g, const Coef<CT>& c, const CT* w, float* sigma1,
+template <class CT, class TIN>
+cudaError_t launch_sigma1(const GridDesc& g, const Coef<CT>& c, const TIN* w, float* sigma1,
                           double* stats, double* scratch, unsigned* ticket, cudaStream_t st,
                           const NuRule* rule, double* sigma1d) {
   const NuRule r = rule ? *rule : NuRule{0.f, 0.f, 0.f, nullptr, nullptr, 0.0, 0.0, 0.0, nullptr, 0};
   const size_t smem = sizeof(CT) * 3 * sgk::NV * sgk::SP;
   static MarchShape<TX, sgk::TY> shape;
   int ctas = 0;
-  cudaError_t e = shape.get(k_sigma1<CT>, smem, g, nullptr, ctas);
+  cudaError_t e = shape.get(k_sigma1<CT, TIN>, smem, g, nullptr, ctas);
   if (e != cudaSuccess) return e;
   if ((size_t)ctas > sigma1_march_ctas_bound(g)) return cudaErrorInvalidConfiguration;
   if (g.batch > sgk::NT) return cudaErrorInvalidConfiguration;
-  e = launch_pdl(k_sigma1<CT>, dim3(ctas), dim3(sgk::NT), smem, st, g, c, w, sigma1, scratch, stats, ticket, r,
+  e = launch_pdl(k_sigma1<CT, TIN>, dim3(ctas), dim3(sgk::NT), smem, st, g, c, w, sigma1, scratch, stats, ticket, r,
                  sigma1d);
   count_launch();
   return e;
 }
-template cudaError_t launch_sigma1<double>(const GridDesc&, const Coef<double>&, const double*, float*,
+template cudaError_t launch_sigma1<float, double>(const GridDesc&, const Coef<float>&, const double*, float*,
+                                                  double*, double*, unsigned*, cudaStream_t, const NuRule*, double*);
+template cudaError_t launch_sigma1<double, double>(const GridDesc&, const Coef<double>&, const double*, float*,
                                            double*, double*, unsigned*, cudaStream_t, const NuRule*, double*);
-template cudaError_t launch_sigma1<float>(const GridDesc&, const Coef<float>&, const float*, float*,
+template cudaError_t launch_sigma1<float, float>(const GridDesc&, const Coef<float>&, const float*, float*,
                                           double*, double*, unsigned*, cudaStream_t, const NuRule*, double*);
 
 template <class CT>
 cudaError_t launch_label(const GridDesc& g, const Coef<CT>& c, const CT* w, const double* lam, float* acc,
                          cudaStream_t st) {
   const long long n = g.cells * g.batch;
-  k_label<CT><<<(unsigned)((n + RB - 1) / RB), RB, 0, st>>>(g, c, w, lam, acc);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_label<CT>, dim3((unsigned)((n + RB - 1) / RB)), dim3(RB), 0, st, g, c, w, lam, acc);
 }
 template cudaError_t launch_label<double>(const GridDesc&, const Coef<double>&, const double*, const double*,
                                           float*, cudaStream_t);
@@ -1139,27 +1142,22 @@ template cudaError_t launch_label<float>(const GridDesc&, const Coef<float>&, co
 cudaError_t launch_nu_rule(const GridDesc& g, const float* sigma1, double lambda, double tau,
                            double limit_nu, float* nu, unsigned* err, cudaStream_t st, bool cap) {
   const long long n = g.cells * g.batch;
-  k_nu_rule<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, sigma1, (float)lambda, (float)tau,
-                                                           (float)limit_nu, nu, err, cap);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_nu_rule, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, n, sigma1, (float)lambda, (float)tau, (float)limit_nu, nu, err, cap);
 }
 
 cudaError_t launch_nu_rule_f64(const GridDesc& g, const double* sigma1, double lambda, double tau,
                                double limit_nu, double* nu, unsigned* err, cudaStream_t st, bool cap) {
   const long long n = g.cells * g.batch;
-  k_nu_rule_f64<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, sigma1, lambda, tau, limit_nu, nu, err, cap);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_nu_rule_f64, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, n, sigma1, lambda, tau, limit_nu, nu, err, cap);
 }
 
 cudaError_t launch_visc_apply(const GridDesc& g, const double* idx2, const double* split, const float* nu,
                               const double* a, double* out, cudaStream_t st) {
   const long long n = g.cells * g.batch;
-  k_visc_apply<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(g, idx2[0], idx2[1], idx2[2], split[0], split[1],
-                                                            split[2], nu, a, out);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_visc_apply, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, g, idx2[0], idx2[1], idx2[2], split[0], split[1], split[2], nu, a, out);
 }
 
 cudaError_t launch_energy(const GridDesc& g, double gamma, double dV, const double* w, const double* lam,
@@ -1187,31 +1185,26 @@ cudaError_t launch_energy_mirrors(const GridDesc& g, double gamma, double dV, co
 cudaError_t launch_dot(const double* a, const double* phi, int nphi, size_t n, double* out,
                        double* scratch, cudaStream_t st) {
   dim3 grid(RG, nphi);
-  k_dot<<<grid, RB, 0, st>>>(a, phi, n, scratch);
   count_launch();
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(k_dot, dim3(grid), dim3(RB), 0, st, a, phi, n, scratch);
   if (e != cudaSuccess) return e;
-  k_sum_partials<<<nphi, RB, 0, st>>>(RG, 1.0, scratch, out, nullptr);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_sum_partials, dim3(nphi), dim3(RB), 0, st, RG, 1.0, scratch, out, nullptr);
 }
 
 cudaError_t launch_combine(const double* theta, const double* phi, int nphi, size_t n, double* s,
                            cudaStream_t st) {
-  k_combine<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(theta, phi, nphi, n, s);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_combine, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, theta, phi, nphi, n, s);
 }
 
 cudaError_t launch_max_wave(const GridDesc& g, double gamma, const double* w, double* out,
                             double* scratch, cudaStream_t st) {
-  k_max_wave<<<RG, RB, 0, st>>>(g, gamma, w, scratch);
   count_launch();
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(k_max_wave, dim3(RG), dim3(RB), 0, st, g, gamma, w, scratch);
   if (e != cudaSuccess) return e;
-  k_max_partials<<<1, RB, 0, st>>>(RG, scratch, out);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_max_partials, dim3(1), dim3(RB), 0, st, RG, scratch, out);
 }
 
 }  // namespace ns
@@ -1219,31 +1212,26 @@ cudaError_t launch_max_wave(const GridDesc& g, double gamma, const double* w, do
 namespace ns {
 cudaError_t launch_scale_boxes(const GridDesc& g, const double* seed, double* field, cudaStream_t st) {
   const long long tot = g.cells * 5 * g.batch;
-  k_scale_boxes<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(g, seed, field);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_scale_boxes, dim3((unsigned)((tot + 255) / 256)), dim3(256), 0, st, g, seed, field);
 }
 
 cudaError_t launch_dot_boxes(const GridDesc& g, const double* field, int comp, const double* phi, int nphi,
                              double* out, double* scratch, cudaStream_t st) {
-  k_dot_boxes<<<dim3(RG, nphi), RB, 0, st>>>(g, field, comp, phi, scratch);
   count_launch();
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(k_dot_boxes, dim3(dim3(RG, nphi)), dim3(RB), 0, st, g, field, comp, phi, scratch);
   if (e != cudaSuccess) return e;
-  k_sum_partials<<<nphi, RB, 0, st>>>(RG, 1.0, scratch, out, nullptr);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_sum_partials, dim3(nphi), dim3(RB), 0, st, RG, 1.0, scratch, out, nullptr);
 }
 
 cudaError_t launch_diff_norms(const double* a, const double* b, size_t n, double* out2, double* scratch,
                               cudaStream_t st) {
-  k_diff_norms<<<RG, RB, 0, st>>>(a, b, n, scratch);
   count_launch();
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(k_diff_norms, dim3(RG), dim3(RB), 0, st, a, b, n, scratch);
   if (e != cudaSuccess) return e;
-  k_sum_partials<<<2, RB, 0, st>>>(RG, 1.0, scratch, out2, nullptr);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_sum_partials, dim3(2), dim3(RB), 0, st, RG, 1.0, scratch, out2, nullptr);
 }
 
 size_t objective_scratch_doubles(const GridDesc& g) {
@@ -1252,8 +1240,7 @@ size_t objective_scratch_doubles(const GridDesc& g) {
 
 cudaError_t launch_to_float(const double* in, float* out, size_t n, cudaStream_t st) {
   const size_t threads = (n + 1) / 2;
-  k_to_float<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(in, out, n);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_to_float, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, st, in, out, n);
 }
 }  // namespace ns

@@ -108,8 +108,8 @@ struct NuRule {
 // null): also writes the viscosity of the sigma_1 rule.
 // sigma1d (may be null; FP64 contexts): sigma_1 in FP64 in place of the float field,
 // with rule->nud the rule's FP64 viscosity.
-template <class CT>
-cudaError_t launch_sigma1(const GridDesc& g, const Coef<CT>& c, const CT* w, float* sigma1,
+template <class CT, class TIN>
+cudaError_t launch_sigma1(const GridDesc& g, const Coef<CT>& c, const TIN* w, float* sigma1,
                           double* stats, double* scratch, unsigned* ticket, cudaStream_t st,
                           const NuRule* rule = nullptr, double* sigma1d = nullptr);
 template <class CT>
