@@ -435,7 +435,13 @@ int ns_create(const ns_params* p, void* stream, ns_ctx** out) {
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < ns_ctx::NSTAGE && e == cudaSuccess; ++i) e = cudaMalloc(&c->stage[i], c->field * esz);
   c->scratch_n = std::max(ns::diag_scratch_doubles(c->g, 256), ns::box_means_scratch_doubles(c->g));
-  if (e == cudaSuccess) e = cudaMalloc(&c->scratch, c->scratch_n * sizeof(double));
+  // behind it the training scratch of an ordinary minibatch (4096 samples, 0.7 MB)
+  const size_t train_n = ns::mlp_train_scratch_floats(4096);
+  if (e == cudaSuccess) e = cudaMalloc(&c->scratch, c->scratch_n * sizeof(double) + train_n * sizeof(float));
+  if (e == cudaSuccess) {
+    c->train_scratch = (float*)(c->scratch + c->scratch_n);
+    c->train_scratch_n = train_n;
+  }
   if (e == cudaSuccess) e = cudaMalloc(&c->err, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMalloc(&c->qbar, sizeof(double) * 5 * p->batch);
   if (e == cudaSuccess) e = cudaMalloc(&c->ticket, sizeof(unsigned) * p->batch);
@@ -482,7 +488,7 @@ void ns_destroy(ns_ctx* c) {
   if (c->ofork) cudaEventDestroy(c->ofork);
   if (c->ojoin) cudaEventDestroy(c->ojoin);
   if (c->ost) cudaStreamDestroy(c->ost);
-  if (c->train_scratch) cudaFree(c->train_scratch);
+  if (c->own_train_scratch) cudaFree(c->own_train_scratch);
   for (cudaEvent_t ev : c->events) cudaEventDestroy(ev);
   free_bounded(c);
   if (c->owns_stream) cudaStreamDestroy(c->st);
@@ -761,10 +767,12 @@ int ns_mlp_train_step(ns_ctx* c, void* net, const float* feat, const float* targ
   if (!c || !net || !feat || !target || !idx || n < 1 || step < 1 || !(lr > 0)) return NS_ERR_ARG;
   const size_t need = ns::mlp_train_scratch_floats(n);
   if (need > c->train_scratch_n) {
-    if (c->train_scratch) cudaFree(c->train_scratch);
-    c->train_scratch = nullptr;
-    c->train_scratch_n = 0;
-    if (cudaMalloc(&c->train_scratch, need * sizeof(float)) != cudaSuccess) return NS_ERR_CUDA;
+    if (c->own_train_scratch) cudaFree(c->own_train_scratch);
+    c->own_train_scratch = nullptr;
+    c->train_scratch = (float*)(c->scratch + c->scratch_n);
+    c->train_scratch_n = ns::mlp_train_scratch_floats(4096);
+    if (cudaMalloc(&c->own_train_scratch, need * sizeof(float)) != cudaSuccess) return NS_ERR_CUDA;
+    c->train_scratch = c->own_train_scratch;
     c->train_scratch_n = need;
   }
   return cuerr(ns::launch_mlp_train_step(net, feat, target, idx, n, step, lr, c->train_scratch, loss, c->st));

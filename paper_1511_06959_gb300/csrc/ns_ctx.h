@@ -47,7 +47,8 @@ struct ns_ctx {
   cudaEvent_t ofork = nullptr, ojoin = nullptr;
   double* oscratch = nullptr;
   unsigned* oticket = nullptr;
-  float* train_scratch = nullptr;    // closure training partials, allocated on first use
+  float* train_scratch = nullptr;    // closure training partials: behind scratch, or own_train_scratch
+  float* own_train_scratch = nullptr;   // for large minibatches, allocated on first use
   size_t train_scratch_n = 0;
   // bounded box (ns_set_boundaries): the padded grid and its workspace
   ns::BcDesc bc{};
