@@ -118,6 +118,7 @@ template <class TO, class TI>
 __global__ void __launch_bounds__(32 * BR) k_bc_embed(GridDesc g, BcDesc bc, int ncomp, double scale,
                                                       const TI* __restrict__ src, TO* __restrict__ dst,
                                                       double* __restrict__ dst2) {
+  pdl_enter();
   const Pad P = pad_of(g, bc);
   const long long rows = (long long)P.nyp * g.nz * ncomp * g.batch;
   const int lane = threadIdx.x & 31;
@@ -140,6 +141,7 @@ __global__ void __launch_bounds__(32 * BR) k_bc_embed(GridDesc g, BcDesc bc, int
 template <class TO, class TI>
 __global__ void __launch_bounds__(32 * BR) k_bc_crop(GridDesc g, BcDesc bc, int ncomp, const TI* __restrict__ src,
                                                      TO* __restrict__ dst) {
+  pdl_enter();
   const Pad P = pad_of(g, bc);
   const long long rows = (long long)g.ny * g.nz * ncomp * g.batch;
   const int lane = threadIdx.x & 31;
@@ -160,6 +162,7 @@ __device__ __forceinline__ void load5(const T* f, long long o, long long stride,
 // the ghost layer of a padded state field, from its interior boundary cells
 template <class T>
 __global__ void k_bc_ghosts(GridDesc g, BcDesc bc, T* __restrict__ W) {
+  pdl_enter();
   const Pad P = pad_of(g, bc);
   // ghost cells per plane: the x columns' interior rows, then the y rows' full width
   const int nxg = P.ix ? 2 * g.ny : 0, nyg = P.iy ? 2 * P.nxp : 0;
@@ -275,7 +278,7 @@ __device__ __forceinline__ void char_pullback(const double wc[5], int side, cons
 // those cells, packed so that all 32 lanes of a warp have one, and the other CTAs the
 // cells of whole rows, leaving out the packed ones.  With every cell in one grid, each
 // row's end cells held two of its three warps for the whole pull-back: 931 us per stage of
-// a 96x48x48 duct (a primal and an adjoint step: 4080 us, now 720 us).
+// a 96x48x48 duct (a primal and an adjoint step: 4070 us, 500 us with this split and the Laplacian below).
 struct EpiArgs {
   const double* gp;
   const double* A;
@@ -296,30 +299,32 @@ __device__ __forceinline__ void epilogue_cell(const GridDesc& g, const Pad& P, c
   const long long r = (long long)z * g.plane + (long long)y * g.nx + x;
   const long long o = (long long)b * 5 * g.cells + r;
   const double sa = e.sa;
-  double a[5];
+  double A[5];
 #pragma unroll
-  for (int k = 0; k < 5; ++k) a[k] = sa * e.A[o + k * g.cells];
+  for (int k = 0; k < 5; ++k) A[k] = e.A[o + k * g.cells];
   if (nu) {
+    // L_nu a = sa (sum_q F_q A_q - (sum_q F_q) A), F_q = (nu + nu_q) / (2 dx_q^2), zero at
+    // closed faces: FP64 operations bind this kernel, and this form takes a third of those
+    // of six scaled differences
     const NU* nb = nu + (long long)b * g.cells;
-    const double nc = (double)nb[r];
-    const long long oxm = r + (x == 0 ? g.nx - 1 : -1), oxq = r + (x == g.nx - 1 ? 1 - g.nx : 1);
-    const long long oym = r + (long long)(y == 0 ? g.ny - 1 : -1) * g.nx,
-                    oyq = r + (long long)(y == g.ny - 1 ? 1 - g.ny : 1) * g.nx;
-    const long long ozm = r + (z == 0 ? g.nz - 1 : -1) * g.plane, ozq = r + (z == g.nz - 1 ? 1 - g.nz : 1) * g.plane;
-    // closed faces pass nothing
-    const double fxm = P.ix && x == 0 ? 0.0 : 0.5 * (nc + (double)nb[oxm]);
-    const double fxq = P.ix && x == g.nx - 1 ? 0.0 : 0.5 * (nc + (double)nb[oxq]);
-    const double fym = P.iy && y == 0 ? 0.0 : 0.5 * (nc + (double)nb[oym]);
-    const double fyq = P.iy && y == g.ny - 1 ? 0.0 : 0.5 * (nc + (double)nb[oyq]);
-    const double fzm = 0.5 * (nc + (double)nb[ozm]), fzq = 0.5 * (nc + (double)nb[ozq]);
+    const double nc = widen(nb[r]);
+    long long q[6] = {r + (x == 0 ? g.nx - 1 : -1), r + (x == g.nx - 1 ? 1 - g.nx : 1),
+                      r + (long long)(y == 0 ? g.ny - 1 : -1) * g.nx, r + (long long)(y == g.ny - 1 ? 1 - g.ny : 1) * g.nx,
+                      r + (z == 0 ? g.nz - 1 : -1) * g.plane, r + (z == g.nz - 1 ? 1 - g.nz : 1) * g.plane};
+    const bool closed[6] = {P.ix && x == 0, P.ix && x == g.nx - 1, P.iy && y == 0, P.iy && y == g.ny - 1, false, false};
+    double F[6], Fs = 0.0;
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+      F[d] = closed[d] ? 0.0 : (nc + widen(nb[q[d]])) * (0.5 * e.i2[d >> 1]);
+      Fs += F[d];
+    }
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
       const double* Ak = e.A + (long long)b * 5 * g.cells + (long long)k * g.cells;
-      const double ac = a[k];
-      const double L = (fxq * (sa * Ak[oxq] - ac) - fxm * (ac - sa * Ak[oxm])) * e.i2[0] +
-                       (fyq * (sa * Ak[oyq] - ac) - fym * (ac - sa * Ak[oym])) * e.i2[1] +
-                       (fzq * (sa * Ak[ozq] - ac) - fzm * (ac - sa * Ak[ozm])) * e.i2[2];
-      gc[k] += e.nus[k == 0 ? 0 : (k == 4 ? 2 : 1)] * L;
+      double L = -Fs * A[k];
+#pragma unroll
+      for (int d = 0; d < 6; ++d) L += F[d] * Ak[q[d]];
+      gc[k] += (sa * e.nus[k == 0 ? 0 : (k == 4 ? 2 : 1)]) * L;
     }
   }
   const long long op = (long long)b * 5 * P.cellsp + (long long)z * P.planep + (long long)(y + P.iy) * P.nxp + x + P.ix;
@@ -335,38 +340,40 @@ __device__ __forceinline__ void epilogue_cell(const GridDesc& g, const Pad& P, c
       e.out[ok] = e.lam[ok] + Gs;
     } else {
       e.G[ok] = Gs;
-      const double an = e.cl * e.lam[ok] + e.cg * gc[k] + e.cs * Gs;
+      double an = e.cl * e.lam[ok] + e.cg * gc[k];
+      if (e.cs != 0.0) an += e.cs * Gs;
       e.a_next[ok] = an;
       seed[op + (long long)k * P.cellsp] = cvt<CT>(an);
     }
-    if (e.sbar) e.sbar[ok] += a[k];
+    if (e.sbar) e.sbar[ok] += sa * A[k];
   }
 }
 
-constexpr int BBT = 32;   // packed boundary cells per CTA: one warp, so that they spread over the SMs
+constexpr int BBT = 64;   // packed boundary cells per CTA: two of its warps, so that they spread over the SMs
 
 template <class CT, class NU>
 __global__ void __launch_bounds__(32 * BR) k_bc_adj_epilogue(GridDesc g, BcDesc bc, EpiArgs e,
                                                              const CT* __restrict__ W, const NU* __restrict__ nu,
                                                              CT* __restrict__ seed, int nbb) {
+  pdl_enter();
   const Pad P = pad_of(g, bc);
   const int lane = threadIdx.x & 31;
   if ((int)blockIdx.x >= nbb) {
-    // whole rows, without the cells next to a boundary
-    const long long rows = (long long)g.ny * g.nz * g.batch, step = (long long)(gridDim.x - nbb) * BR;
-    for (long long r = (long long)(blockIdx.x - nbb) * BR + (threadIdx.x >> 5); r < rows; r += step) {
-      const int y = (int)(r % g.ny);
+    // 32-cell pieces of rows, one per warp, without the cells next to a boundary
+    const int pieces = (g.nx + 31) / 32;
+    const long long jobs = (long long)pieces * g.ny * g.nz * g.batch, step = (long long)(gridDim.x - nbb) * BR;
+    for (long long j = (long long)(blockIdx.x - nbb) * BR + (threadIdx.x >> 5); j < jobs; j += step) {
+      const long long r = j / pieces;
+      const int x = (int)(j - r * pieces) * 32 + lane;
       const long long q = r / g.ny;
+      const int y = (int)(r - q * g.ny);
       const int z = (int)(q % g.nz), b = (int)(q / g.nz);
-      if (P.iy && (y == 0 || y == g.ny - 1)) continue;
+      if (x >= g.nx || (P.iy && (y == 0 || y == g.ny - 1)) || (P.ix && (x == 0 || x == g.nx - 1))) continue;
       const double* gr = e.gp + (long long)b * 5 * P.cellsp + (long long)z * P.planep +
                          (long long)(y + P.iy) * P.nxp + P.ix;
-      for (int x = lane; x < g.nx; x += 32) {
-        if (P.ix && (x == 0 || x == g.nx - 1)) continue;
-        double gc[5];
-        load5(gr, x, P.cellsp, gc);
-        epilogue_cell<CT, NU>(g, P, e, nu, seed, b, x, y, z, gc);
-      }
+      double gc[5];
+      load5(gr, x, P.cellsp, gc);
+      epilogue_cell<CT, NU>(g, P, e, nu, seed, b, x, y, z, gc);
     }
     return;
   }
@@ -432,7 +439,7 @@ __global__ void __launch_bounds__(32 * BR) k_bc_adj_epilogue(GridDesc g, BcDesc 
   epilogue_cell<CT, NU>(g, P, e, nu, seed, b, x, y, z, gc);
 }
 
-constexpr int BB = 256;
+constexpr int BB = 64;   // ghost cells per CTA: few, so that they spread over the SMs
 
 unsigned blocks_for(long long n) {
   long long b = (n + BB - 1) / BB;
@@ -456,25 +463,23 @@ template <class TO, class TI>
 cudaError_t launch_bc_embed(const GridDesc& g, const BcDesc& bc, int ncomp, double scale, const TI* src, TO* dst,
                             cudaStream_t st, double* dst2) {
   const long long rows = (long long)(g.ny + 2 * bc.walls) * g.nz * ncomp * g.batch;
-  k_bc_embed<TO, TI><<<blocks_for_rows(rows), 32 * BR, 0, st>>>(g, bc, ncomp, scale, src, dst, dst2);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_bc_embed<TO, TI>, dim3(blocks_for_rows(rows)), dim3(32 * BR), 0, st, g, bc, ncomp, scale, src, dst,
+                    dst2);
 }
 
 template <class TO, class TI>
 cudaError_t launch_bc_crop(const GridDesc& g, const BcDesc& bc, int ncomp, const TI* src, TO* dst, cudaStream_t st) {
   const long long rows = (long long)g.ny * g.nz * ncomp * g.batch;
-  k_bc_crop<TO, TI><<<blocks_for_rows(rows), 32 * BR, 0, st>>>(g, bc, ncomp, src, dst);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_bc_crop<TO, TI>, dim3(blocks_for_rows(rows)), dim3(32 * BR), 0, st, g, bc, ncomp, src, dst);
 }
 
 template <class T>
 cudaError_t launch_bc_ghosts(const GridDesc& g, const BcDesc& bc, T* W, cudaStream_t st) {
   const long long per = (long long)((bc.inout ? 2 * g.ny : 0) + (bc.walls ? 2 * (g.nx + 2 * bc.inout) : 0)) * g.nz;
-  k_bc_ghosts<T><<<blocks_for(per * g.batch), BB, 0, st>>>(g, bc, W);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_bc_ghosts<T>, dim3(blocks_for(per * g.batch)), dim3(BB), 0, st, g, bc, W);
 }
 
 template <class CT, class NU>
@@ -490,10 +495,10 @@ cudaError_t launch_bc_adj_epilogue(const GridDesc& g, const BcDesc& bc, const Bc
   const long long cells = (ncol * g.ny + nrow * (g.nx - ncol)) * g.nz * g.batch;   // next to a boundary
   const long long nbb = (cells + BBT - 1) / BBT;
   if (nbb > (1LL << 30)) return cudaErrorInvalidConfiguration;
-  const unsigned rows = blocks_for_rows((long long)g.ny * g.nz * g.batch);
-  k_bc_adj_epilogue<CT, NU><<<(unsigned)nbb + rows, 32 * BR, 0, st>>>(g, bc, a, W, nu, seed, (int)nbb);
+  const unsigned rows = blocks_for_rows((long long)((g.nx + 31) / 32) * g.ny * g.nz * g.batch);
   count_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_bc_adj_epilogue<CT, NU>, dim3((unsigned)nbb + rows), dim3(32 * BR), 0, st, g, bc, a, W, nu, seed,
+                    (int)nbb);
 }
 
 template cudaError_t launch_bc_embed<double, double>(const GridDesc&, const BcDesc&, int, double, const double*,
