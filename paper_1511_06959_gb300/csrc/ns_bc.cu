@@ -278,7 +278,7 @@ __device__ __forceinline__ void char_pullback(const double wc[5], int side, cons
 // those cells, packed so that all 32 lanes of a warp have one, and the other CTAs the
 // cells of whole rows, leaving out the packed ones.  With every cell in one grid, each
 // row's end cells held two of its three warps for the whole pull-back: 931 us per stage of
-// a 96x48x48 duct (a primal and an adjoint step: 4070 us, 500 us with this split and the Laplacian below).
+// a 96x48x48 duct (a primal and an adjoint step: 4070 us, 511 us with this split and the Laplacian below).
 struct EpiArgs {
   const double* gp;
   const double* A;
@@ -303,27 +303,24 @@ __device__ __forceinline__ void epilogue_cell(const GridDesc& g, const Pad& P, c
 #pragma unroll
   for (int k = 0; k < 5; ++k) A[k] = e.A[o + k * g.cells];
   if (nu) {
-    // L_nu a = sa (sum_q F_q A_q - (sum_q F_q) A), F_q = (nu + nu_q) / (2 dx_q^2), zero at
-    // closed faces: FP64 operations bind this kernel, and this form takes a third of those
-    // of six scaled differences
+    // L_nu a = sa sum_q F_q (A_q - A), F_q = (nu + nu_q) / (2 dx_q^2), zero at closed faces:
+    // FP64 operations bind this kernel, so the weights are formed once per cell and the
+    // seed's scale is applied once per component
     const NU* nb = nu + (long long)b * g.cells;
     const double nc = widen(nb[r]);
     long long q[6] = {r + (x == 0 ? g.nx - 1 : -1), r + (x == g.nx - 1 ? 1 - g.nx : 1),
                       r + (long long)(y == 0 ? g.ny - 1 : -1) * g.nx, r + (long long)(y == g.ny - 1 ? 1 - g.ny : 1) * g.nx,
                       r + (z == 0 ? g.nz - 1 : -1) * g.plane, r + (z == g.nz - 1 ? 1 - g.nz : 1) * g.plane};
     const bool closed[6] = {P.ix && x == 0, P.ix && x == g.nx - 1, P.iy && y == 0, P.iy && y == g.ny - 1, false, false};
-    double F[6], Fs = 0.0;
+    double F[6];
 #pragma unroll
-    for (int d = 0; d < 6; ++d) {
-      F[d] = closed[d] ? 0.0 : (nc + widen(nb[q[d]])) * (0.5 * e.i2[d >> 1]);
-      Fs += F[d];
-    }
+    for (int d = 0; d < 6; ++d) F[d] = closed[d] ? 0.0 : (nc + widen(nb[q[d]])) * (0.5 * e.i2[d >> 1]);
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
       const double* Ak = e.A + (long long)b * 5 * g.cells + (long long)k * g.cells;
-      double L = -Fs * A[k];
+      double L = 0.0;
 #pragma unroll
-      for (int d = 0; d < 6; ++d) L += F[d] * Ak[q[d]];
+      for (int d = 0; d < 6; ++d) L += F[d] * (Ak[q[d]] - A[k]);
       gc[k] += (sa * e.nus[k == 0 ? 0 : (k == 4 ? 2 : 1)]) * L;
     }
   }
