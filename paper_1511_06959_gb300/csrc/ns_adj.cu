@@ -604,7 +604,10 @@ __global__ void __launch_bounds__(NT, AdjMinBlocks<CT, ROE>::value) k_adj_stage(
   const int tid = threadIdx.x;
   const int tx = tid % TX, ty = tid / TX;
   int b, x0, y0, kz0, kz1;
-  march_range<TX, TY>(g, b, x0, y0, kz0, kz1);
+  // (the FP32 Roe product rounds a range's first z-face in code of its own, so its bits
+  // depend on where the ranges are cut: it keeps one rule for them)
+  if constexpr (ROE) march_even<TX, TY>(g, b, x0, y0, kz0, kz1);
+  else if (!march_range<TX, TY>(g, b, x0, y0, kz0, kz1)) return;
   const int gx = x0 + tx, gy = y0 + ty;
   const bool valid = gx < g.nx && gy < g.ny;
   const int cp = valid ? gy * g.nx + gx : 0;   // the thread's cell within a plane
@@ -1031,22 +1034,23 @@ static cudaError_t launch_adj_flat(const GridDesc& g, const Coef<CT>& c, const A
 }
 
 template <class CT, class TIN, class TA, class TST, bool ROE>
-static cudaError_t launch_adj_variant(const GridDesc& g, const Coef<CT>& c, const AdjArgs<TIN, TA, TST>& a,
+static cudaError_t launch_adj_flat_rows(const GridDesc& g, const Coef<CT>& c, const AdjArgs<TIN, TA, TST>& a,
+                                       cudaStream_t st) {
+  return flat_rows(g) == 1 ? launch_adj_flat<CT, TIN, TA, TST, ROE, 1>(g, c, a, st)
+                           : launch_adj_flat<CT, TIN, TA, TST, ROE, 4>(g, c, a, st);
+}
+
+template <class CT, class TIN, class TA, class TST, bool ROE>
+static cudaError_t launch_adj_march(const GridDesc& g, const Coef<CT>& c, const AdjArgs<TIN, TA, TST>& a,
                                      cudaStream_t st) {
-  // 2D boxes; the FP32 Roe product stays with the marching kernel, whose rounding of the
-  // dissipation's transpose the flat kernel does not reproduce
-  if constexpr (!(ROE && std::is_same<CT, float>::value)) {
-    if (g.nz == 1)
-      return flat_rows(g) == 1 ? launch_adj_flat<CT, TIN, TA, TST, ROE, 1>(g, c, a, st)
-                               : launch_adj_flat<CT, TIN, TA, TST, ROE, 4>(g, c, a, st);
-  }
   const size_t smem = adj_smem_bytes<CT, ROE>();
   auto kern = k_adj_stage<CT, TIN, TA, TST, ROE>;
   static MarchShape<TX, TY> shape;
   int ctas = 0;
-  cudaError_t e = shape.get(kern, smem, g, "NS_ADJ_CTAS", ctas);
+  GridDesc gm = g;
+  cudaError_t e = shape.get_ranges(kern, smem, gm, "NS_ADJ_CTAS", ctas, !ROE, ROE && sizeof(CT) == 4);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(kern, dim3(ctas), dim3(NT), smem, st, g, c, a);
+  e = launch_pdl(kern, dim3(ctas), dim3(NT), smem, st, gm, c, a);
   count_launch();
   return e;
 }
@@ -1056,8 +1060,15 @@ static cudaError_t launch_adj_variant(const GridDesc& g, const Coef<CT>& c, cons
 template <class CT, class TIN, class TA, class TST>
 cudaError_t launch_adj_stage(const GridDesc& g, const Coef<CT>& c, const AdjArgs<TIN, TA, TST>& a,
                              cudaStream_t st) {
-  return c.roe ? adjk::launch_adj_variant<CT, TIN, TA, TST, true>(g, c, a, st)
-               : adjk::launch_adj_variant<CT, TIN, TA, TST, false>(g, c, a, st);
+  // 2D boxes; the FP32 Roe product stays with the marching kernel, whose rounding of the
+  // dissipation's transpose the flat kernel does not reproduce
+  if (g.nz == 1 && !c.roe) return adjk::launch_adj_flat_rows<CT, TIN, TA, TST, false>(g, c, a, st);
+  if constexpr (std::is_same<CT, double>::value) {
+    if (g.nz == 1) return adjk::launch_adj_flat_rows<CT, TIN, TA, TST, true>(g, c, a, st);
+  }
+  if (c.roe) return adjk::launch_adj_march<CT, TIN, TA, TST, true>(g, c, a, st);
+  return adjk::launch_adj_march<CT, TIN, TA, TST, false>(g, c, a, st);
+
 }
 
 template cudaError_t launch_adj_stage<double, double, double, double>(

@@ -7,11 +7,14 @@
 // computed once; periodic wrap is resolved when a plane is loaded, so every shared
 // position holds a valid cell even when the box is smaller than the tile.
 //
-// Work split: the CTAs of a launch, as many as the kernel has resident slots on the
-// device (occupancy calculator x SMs), are dealt out to the tile columns as evenly as
-// integers allow (column c gets floor((c+1)G/C) - floor(cG/C) of the G CTAs), and each
-// column's planes are cut into that many ranges whose lengths differ by at most one.
-// One wave of CTAs then covers the grid with every SM holding the same number of CTAs.
+// Work split (MarchShape): a launch has as many CTAs as the kernel has resident slots on
+// the device (occupancy calculator x SMs), so that one wave covers the grid, and shares
+// the planes of all tile columns among them.  The FP64 kernels, which have registers to
+// spare, lay the columns end to end, with MARCH_GAP units between two columns for the cost
+// of starting one, and cut that into equal pieces; a CTA marches its piece, range by range
+// where it spans the end of a column (March).  In the FP32 kernels that outer loop costs
+// registers they do not have (the adjoint stage spilled and took 15% longer): there a CTA
+// marches one range (march_range), chosen as get_ranges says.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -36,14 +39,47 @@ struct GridDesc {
   long long plane;     // nx * ny
   long long cells;     // nx * ny * nz  (one box)
   unsigned* dbg_err;   // sticky error word for the bounds checks of debug builds (may be null)
+  int split;           // split of a one-range-per-CTA march (set for each launch)
 };
 
-constexpr int MIN_PLANES = 4;   // fewest planes per CTA range (bounds the priming share)
+constexpr int MARCH_SPLIT = 8;  // most ranges per column in whole waves
+constexpr int MARCH_GAP = 2;    // planes' worth of starting a range: priming its three planes
 
-// Plane range of this CTA for tiles of TXK x TYK columns (see the file comment).
+// The ranges of this CTA's piece, one tile column after the other, for tiles of TXK x TYK
+// columns (see the file comment).  The state is the last column alone: a march keeps one
+// register for it, and the piece's ends are formed again at each column.  128x64x64, FP64
+// primal step: 1021 us with each column cut into whole ranges (up to 16 planes, the mean
+// being 13.5), 915 us in pieces.
 template <int TXK, int TYK>
-__device__ __forceinline__ void march_range(const GridDesc& g, int& b, int& x0, int& y0, int& kz0,
-                                            int& kz1) {
+struct March {
+  int col = -1;
+  // the next range: box b, tile origin, planes [kz0, kz1); false when the piece is done
+  __device__ __forceinline__ bool next(const GridDesc& g, int& b, int& x0, int& y0, int& kz0, int& kz1) {
+    const int ncx = (g.nx + TXK - 1) / TXK, ncy = (g.ny + TYK - 1) / TYK, len = g.nz + MARCH_GAP;
+    const long long T = (long long)ncx * ncy * g.batch * len - MARCH_GAP;
+    const long long u0 = T * blockIdx.x / gridDim.x, u1 = T * (blockIdx.x + 1) / gridDim.x;
+    if (col < 0) {
+      col = (int)(u0 / len);
+      if (u0 - (long long)col * len >= g.nz) ++col;   // the piece begins in a gap
+    } else {
+      ++col;
+    }
+    const long long start = (long long)col * len;
+    if (start >= u1) return false;
+    kz0 = u0 > start ? (int)(u0 - start) : 0;
+    kz1 = u1 - start < g.nz ? (int)(u1 - start) : g.nz;
+    x0 = (col % ncx) * TXK;
+    const int r = col / ncx;
+    y0 = (r % ncy) * TYK;
+    b = r / ncy;
+    return true;
+  }
+};
+
+// One range per CTA, the CTAs dealt out to the tile columns as evenly as integers allow and
+// each column's planes cut into that many ranges.
+template <int TXK, int TYK>
+__device__ __forceinline__ void march_even(const GridDesc& g, int& b, int& x0, int& y0, int& kz0, int& kz1) {
   const int ncx = (g.nx + TXK - 1) / TXK, ncy = (g.ny + TYK - 1) / TYK;
   const long long C = (long long)ncx * ncy * g.batch, G = gridDim.x, i = blockIdx.x;
   const int col = (int)(((i + 1) * C - 1) / G);
@@ -57,17 +93,59 @@ __device__ __forceinline__ void march_range(const GridDesc& g, int& b, int& x0, 
   b = r / ncy;
 }
 
-// Launch shape of a plane-marching kernel (see the file comment): the CTA count.  The resident slots come from the occupancy calculator with
-// the kernel's dynamic shared memory and are cached per device; the kernel's dynamic
-// shared-memory limit is raised once.  The environment variable `env`, when set to a
-// positive count, overrides the CTA count.  At least one CTA per tile column, at most
-// nz / MIN_PLANES per column.
+// One range per CTA under the split that MarchShape::get_ranges chose: even (g.split = 0),
+// or g.split equal pieces of the columns laid end to end (see March), where CTA i < g.split
+// takes the first range of piece i and the CTAs after them the beginnings of the columns
+// that a piece reaches from the column before.  False, with an empty range of column 0,
+// when there is none.
+template <int TXK, int TYK>
+__device__ __forceinline__ bool march_range(const GridDesc& g, int& b, int& x0, int& y0, int& kz0, int& kz1) {
+  if (g.split == 0) {
+    march_even<TXK, TYK>(g, b, x0, y0, kz0, kz1);
+    return true;
+  }
+  const int ncx = (g.nx + TXK - 1) / TXK, ncy = (g.ny + TYK - 1) / TYK;
+  const long long len = g.nz + MARCH_GAP, T = (long long)ncx * ncy * g.batch * len - MARCH_GAP, G = g.split,
+                  i = blockIdx.x;
+  int col;
+  long long start, u0, u1;   // the column's start and the range's ends
+  if (i < G) {
+    u0 = T * i / G;
+    u1 = T * (i + 1) / G;
+    col = (int)(u0 / len);
+    if (u0 - col * len >= g.nz) ++col;   // the piece begins in a gap
+    start = col * len;
+    if (u0 < start) u0 = start;
+  } else {
+    col = (int)(i - G) + 1;
+    start = u0 = col * len;
+    const long long q = ((start - MARCH_GAP) * G - 1) / T;   // piece of the last plane before
+    u1 = T * (q + 1) / G;
+  }
+  kz0 = (int)(u0 - start);
+  kz1 = u1 - start < g.nz ? (int)(u1 - start) : g.nz;
+  if (kz0 >= kz1) {
+    b = x0 = y0 = kz0 = kz1 = 0;
+    return false;
+  }
+  x0 = (col % ncx) * TXK;
+  const int r = col / ncx;
+  y0 = (r % ncy) * TYK;
+  b = r / ncy;
+  return true;
+}
+
+// Launch shape of a plane-marching kernel: the CTA count (see the file comment).  The
+// resident slots come from the occupancy calculator with the kernel's dynamic shared memory
+// and are cached per device; the kernel's dynamic shared-memory limit is raised once.  The
+// environment variable `env`, when set to a positive count, overrides the number of slots.
+// At most one CTA per plane of a column.
 template <int TXK, int TYK>
 struct MarchShape {
   static constexpr int NTK = TXK * TYK;
   int per_dev[16] = {0};
   template <class K>
-  cudaError_t get(K kern, size_t smem, const GridDesc& g, const char* env, int& ctas) {
+  cudaError_t slots_of(K kern, size_t smem, const char* env, long long& n) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -83,15 +161,66 @@ struct MarchShape {
       slots = (per_sm > 0 ? per_sm : 1) * sms;
       if (dev >= 0 && dev < 16) per_dev[dev] = slots;
     }
-    const long long cols = (long long)((g.nx + TXK - 1) / TXK) * ((g.ny + TYK - 1) / TYK) * g.batch;
-    long long n = slots;
+    n = slots;
     const char* ov = env ? getenv(env) : nullptr;
     if (ov && atoll(ov) > 0) n = atoll(ov);
-    const long long most = cols * (g.nz / MIN_PLANES > 1 ? g.nz / MIN_PLANES : 1);
-    if (n > most) n = most;
-    if (n < cols) n = cols;
-    if (n > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    ctas = (int)n;
+    return cudaSuccess;
+  }
+  static long long columns(const GridDesc& g) {
+    return (long long)((g.nx + TXK - 1) / TXK) * ((g.ny + TYK - 1) / TYK) * g.batch;
+  }
+  // kernels that march pieces (March)
+  template <class K>
+  cudaError_t get(K kern, size_t smem, const GridDesc& g, const char* env, int& ctas) {
+    long long n = 0;
+    const cudaError_t e = slots_of(kern, smem, env, n);
+    if (e != cudaSuccess) return e;
+    const long long cols = columns(g);
+    if (cols > (1LL << 26)) return cudaErrorInvalidConfiguration;
+    ctas = (int)(n < cols * g.nz ? n : cols * g.nz);
+    return cudaSuccess;
+  }
+  // kernels that march one range per CTA: also sets g.split for march_range (pieces: the
+  // kernel takes the split into pieces; otherwise it uses march_even; fixed_cuts: see
+  // k_adj_stage).  The pieces' second
+  // parts are further CTAs that start as slots fall free; they pay while there are few of
+  // them (one per column) and the pieces are longer than a range's priming.  128x64x64,
+  // adjoint step: 211 us even, 203 us in pieces; with 144 columns on 304 slots (eight
+  // 96x48x48 boxes) 605 us even, 781 us in pieces.  Even ranges are as many as the slots or,
+  // when the columns are too many for that, the number of ranges per column with the
+  // shortest whole waves: the 512 columns of a 512x256x128 box took 2310 us per primal step
+  // in one range each (456 slots: a second wave with 56 CTAs), 1850 us in this split.
+  template <class K>
+  cudaError_t get_ranges(K kern, size_t smem, GridDesc& g, const char* env, int& ctas, bool pieces = true,
+                         bool fixed_cuts = false) {
+    long long n = 0;
+    const cudaError_t e = slots_of(kern, smem, env, n);
+    if (e != cudaSuccess) return e;
+    const long long cols = columns(g);
+    if (cols > (1LL << 26)) return cudaErrorInvalidConfiguration;
+    g.split = 0;
+    if (fixed_cuts) {
+      // one wave of even ranges of at least four planes
+      const long long most = cols * (g.nz / 4 > 1 ? g.nz / 4 : 1);
+      ctas = (int)(n < cols ? cols : (n < most ? n : most));
+      return cudaSuccess;
+    }
+    if (pieces && cols <= n / 8 && cols * g.nz >= 4 * n) {
+      g.split = (int)n;
+      ctas = (int)(n + cols - 1);
+      return cudaSuccess;
+    }
+    // planes a slot marches: one wave of all slots, or whole waves of m ranges per column
+    long long best = cols <= n ? (g.nz + n / cols - 1) / (n / cols) + MARCH_GAP : 1LL << 62, count = n;
+    const int most = g.nz < MARCH_SPLIT ? g.nz : MARCH_SPLIT;
+    for (int m = 1; m <= most; ++m) {
+      const long long cost = ((cols * m + n - 1) / n) * ((g.nz + m - 1) / m + MARCH_GAP);
+      if (cost < best) {
+        best = cost;
+        count = cols * m;
+      }
+    }
+    ctas = (int)(count < cols * g.nz ? count : cols * g.nz);
     return cudaSuccess;
   }
 };

@@ -493,7 +493,7 @@ static_assert(SP <= 2 * NT, "a plane must fit two load rounds");
 size_t sigma1_march_ctas_bound(const GridDesc& g) {
   // the padded (bounded) box has one more column on each side
   const long long cols = (long long)((g.nx + 2 + TX - 1) / TX) * ((g.ny + 2 + sgk::TY - 1) / sgk::TY) * g.batch;
-  return (size_t)(cols > 2048 ? cols : 2048);
+  return (size_t)(MARCH_SPLIT * cols > 2048 ? MARCH_SPLIT * cols : 2048);
 }
 
 // TIN: the state's type; a mixed-precision context's FP64 state is rounded as it is loaded
@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(sgk::NT, sizeof(CT) == 4 ? 4 : 1) k_sigma1(Gri
   const int tid = threadIdx.x;
   const int tx = tid % TX, ty = tid / TX;
   int b, x0, y0, kz0, kz1;
-  march_range<TX, TY>(g, b, x0, y0, kz0, kz1);
+  march_range<TX, TY>(g, b, x0, y0, kz0, kz1);   // (an empty range adds zeros to the statistics)
   const int gx = x0 + tx, gy = y0 + ty;
   const bool valid = gx < g.nx && gy < g.ny;
   const int cp = valid ? gy * g.nx + gx : 0;
@@ -1111,11 +1111,12 @@ cudaError_t launch_sigma1(const GridDesc& g, const Coef<CT>& c, const TIN* w, fl
   const size_t smem = sizeof(CT) * 3 * sgk::NV * sgk::SP;
   static MarchShape<TX, sgk::TY> shape;
   int ctas = 0;
-  cudaError_t e = shape.get(k_sigma1<CT, TIN>, smem, g, nullptr, ctas);
+  GridDesc gm = g;
+  cudaError_t e = shape.get_ranges(k_sigma1<CT, TIN>, smem, gm, nullptr, ctas);
   if (e != cudaSuccess) return e;
   if ((size_t)ctas > sigma1_march_ctas_bound(g)) return cudaErrorInvalidConfiguration;
   if (g.batch > sgk::NT) return cudaErrorInvalidConfiguration;
-  e = launch_pdl(k_sigma1<CT, TIN>, dim3(ctas), dim3(sgk::NT), smem, st, g, c, w, sigma1, scratch, stats, ticket, r,
+  e = launch_pdl(k_sigma1<CT, TIN>, dim3(ctas), dim3(sgk::NT), smem, st, gm, c, w, sigma1, scratch, stats, ticket, r,
                  sigma1d);
   count_launch();
   return e;

@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(RB) k_box_means_final(int nblk, double inv_cel
 // ------------------------------------------------------------------------------------
 // features
 // ------------------------------------------------------------------------------------
-// One CTA takes TX x FY columns and a range of planes (march_range) and keeps 1/rho and
+// One CTA takes TX x FY columns and ranges of planes (March) and keeps 1/rho and
 // rho u of three planes with a one-cell halo in a shared-memory ring, so each cell's state is loaded
 // and divided once per tile instead of seven times; a warp's 32 x 16 features go out
 // through shared memory as whole lines.  1.77 M cells in eight boxes: 115 us with a thread
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(fk::NT) k_features(GridDesc g, Coef<float> c, 
   float* sO = sQ + 3 * 4 * SP;                       // [NT][OS]
   const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX, lane = tid & 31;
   int b, x0, y0, kz0, kz1;
-  march_range<TX, FY>(g, b, x0, y0, kz0, kz1);
+  if (!march_range<TX, FY>(g, b, x0, y0, kz0, kz1)) return;
   const int gx = x0 + tx, gy = y0 + ty;
   const bool valid = gx < g.nx && gy < g.ny;
   const int cp = valid ? gy * g.nx + gx : 0;
@@ -796,10 +796,11 @@ cudaError_t launch_features(const GridDesc& g, const Coef<float>& c, const TIN* 
                             float* feat, cudaStream_t st) {
   static MarchShape<TX, fk::FY> shape;
   int ctas = 0;
-  cudaError_t e = shape.get(k_features<TIN>, fk::smem, g, nullptr, ctas);
+  GridDesc gm = g;
+  cudaError_t e = shape.get_ranges(k_features<TIN>, fk::smem, gm, nullptr, ctas);
   if (e != cudaSuccess) return e;
   count_launch();
-  return launch_pdl(k_features<TIN>, dim3(ctas), dim3(fk::NT), fk::smem, st, g, c, w, qbar, feat);
+  return launch_pdl(k_features<TIN>, dim3(ctas), dim3(fk::NT), fk::smem, st, gm, c, w, qbar, feat);
 }
 template cudaError_t launch_box_means<double>(const GridDesc&, double, const double*, double*, double*, cudaStream_t);
 template cudaError_t launch_box_means<float>(const GridDesc&, double, const float*, double*, double*, cudaStream_t);

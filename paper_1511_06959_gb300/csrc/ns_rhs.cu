@@ -267,11 +267,11 @@ __global__ void __launch_bounds__(NT, RhsMinBlocks<CT, ROE>::value) k_rhs_stage(
   CT* sQ = reinterpret_cast<CT*>(smem_raw);          // [3][5][SP]
   CT* sFX = sQ + 3 * 5 * SP;                          // [5][TY][TX+1]
   CT* sFY = sFX + 5 * TY * (TX + 1);                  // [5][TY+1][TX]
+  Loader<CT, TIN> in{a.W, a.Wd, &g};
   const int tid = threadIdx.x;
   const int tx = tid % TX, ty = tid / TX;
-  Loader<CT, TIN> in{a.W, a.Wd, &g};
   int b, x0, y0, kz0, kz1;
-  march_range<TX, TY>(g, b, x0, y0, kz0, kz1);
+  if (!march_range<TX, TY>(g, b, x0, y0, kz0, kz1)) return;
   const int gx = x0 + tx, gy = y0 + ty;
   const bool valid = gx < g.nx && gy < g.ny;
   const int cp = valid ? gy * g.nx + gx : 0;        // the thread's cell within a plane
@@ -554,20 +554,23 @@ static cudaError_t launch_rhs_flat(const GridDesc& g, const Coef<CT>& c, const S
 }
 
 template <class CT, class TIN, class TST, bool ROE>
-static cudaError_t launch_rhs_variant(const GridDesc& g, const Coef<CT>& c, const StageArgs<TIN, TST>& a,
-                                     cudaStream_t st) {
-  if constexpr (!std::is_same<CT, Dual>::value) {
-    if (g.nz == 1)
-      return flat_rows(g) == 1 ? launch_rhs_flat<CT, TIN, TST, ROE, 1>(g, c, a, st)
-                               : launch_rhs_flat<CT, TIN, TST, ROE, 4>(g, c, a, st);
-  }
+static cudaError_t launch_rhs_flat_rows(const GridDesc& g, const Coef<CT>& c, const StageArgs<TIN, TST>& a,
+                                       cudaStream_t st) {
+  return flat_rows(g) == 1 ? launch_rhs_flat<CT, TIN, TST, ROE, 1>(g, c, a, st)
+                           : launch_rhs_flat<CT, TIN, TST, ROE, 4>(g, c, a, st);
+}
+
+template <class CT, class TIN, class TST, bool ROE>
+static cudaError_t launch_rhs_march(const GridDesc& g, const Coef<CT>& c, const StageArgs<TIN, TST>& a,
+                                   cudaStream_t st) {
   const size_t smem = rhs_smem_bytes<CT>();
   auto kern = rk::k_rhs_stage<CT, TIN, TST, ROE>;
   static MarchShape<TX, rk::TY> shape;
   int ctas = 0;
-  cudaError_t e = shape.get(kern, smem, g, "NS_RHS_CTAS", ctas);
+  GridDesc gm = g;
+  cudaError_t e = shape.get_ranges(kern, smem, gm, "NS_RHS_CTAS", ctas);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(kern, dim3(ctas), dim3(rk::NT), smem, st, g, c, a);
+  e = launch_pdl(kern, dim3(ctas), dim3(rk::NT), smem, st, gm, c, a);
   count_launch();
   return e;
 }
@@ -575,8 +578,13 @@ static cudaError_t launch_rhs_variant(const GridDesc& g, const Coef<CT>& c, cons
 template <class CT, class TIN, class TST>
 cudaError_t launch_rhs_stage(const GridDesc& g, const Coef<CT>& c, const StageArgs<TIN, TST>& a,
                              cudaStream_t st) {
-  return c.roe ? launch_rhs_variant<CT, TIN, TST, true>(g, c, a, st)
-               : launch_rhs_variant<CT, TIN, TST, false>(g, c, a, st);
+  if constexpr (!std::is_same<CT, Dual>::value) {
+    if (g.nz == 1 && !c.roe) return launch_rhs_flat_rows<CT, TIN, TST, false>(g, c, a, st);
+    if (g.nz == 1) return launch_rhs_flat_rows<CT, TIN, TST, true>(g, c, a, st);
+  }
+  if (c.roe) return launch_rhs_march<CT, TIN, TST, true>(g, c, a, st);
+  return launch_rhs_march<CT, TIN, TST, false>(g, c, a, st);
+
 }
 
 template cudaError_t launch_rhs_stage<double, double, double>(const GridDesc&, const Coef<double>&,
