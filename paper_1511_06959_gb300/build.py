@@ -20,7 +20,7 @@ BUILD = os.path.join(HERE, "_build")
 # NS_ADJOINT_LIB=<OUT_DEBUG>
 OUT_DEBUG = os.path.join(HERE, "libns_adjoint_debug.so")
 BUILD_DEBUG = os.path.join(HERE, "_build_debug")
-SOURCES = ["ns_rhs.cu", "ns_adj.cu", "ns_diag.cu", "ns_api.cu", "ns_sweep.cu", "ns_noalloc.cu", "ns_mlp.cu",
+SOURCES = ["ns_rhs.cu", "ns_adj.cu", "ns_f64.cu", "ns_diag.cu", "ns_api.cu", "ns_sweep.cu", "ns_noalloc.cu", "ns_mlp.cu",
            "ns_lambda.cu", "ns_probe.cu", "ns_bc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # Single-precision division and square root in the fast form (-prec-div/-prec-sqrt off):

@@ -1067,8 +1067,8 @@ cudaError_t launch_adj_stage(const GridDesc& g, const Coef<CT>& c, const AdjArgs
     if (g.nz == 1) return adjk::launch_adj_flat_rows<CT, TIN, TA, TST, true>(g, c, a, st);
   }
   if (c.roe) return adjk::launch_adj_march<CT, TIN, TA, TST, true>(g, c, a, st);
-  return adjk::launch_adj_march<CT, TIN, TA, TST, false>(g, c, a, st);
-
+  if constexpr (std::is_same<CT, double>::value) return launch_adj_f64(g, c, a, st);
+  else return adjk::launch_adj_march<CT, TIN, TA, TST, false>(g, c, a, st);
 }
 
 template cudaError_t launch_adj_stage<double, double, double, double>(

@@ -77,6 +77,12 @@ template <class CT, class TIN, class TA, class TST>
 cudaError_t launch_adj_stage(const GridDesc& g, const Coef<CT>& c, const AdjArgs<TIN, TA, TST>& a,
                              cudaStream_t st);
 
+// the same in FP64 on 3D boxes with the central flux (ns_f64.cu)
+cudaError_t launch_rhs_f64(const GridDesc& g, const Coef<double>& c, const StageArgs<double, double>& a,
+                           cudaStream_t st);
+cudaError_t launch_adj_f64(const GridDesc& g, const Coef<double>& c, const AdjArgs<double, double, double>& a,
+                           cudaStream_t st);
+
 // diagnostics and reductions (ns_diag.cu); `scratch` is context workspace of at
 // least diag_scratch_doubles(g) doubles, `err` the sticky device error word
 size_t diag_scratch_doubles(const GridDesc& g, int nphi);

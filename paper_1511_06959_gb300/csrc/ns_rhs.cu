@@ -583,8 +583,8 @@ cudaError_t launch_rhs_stage(const GridDesc& g, const Coef<CT>& c, const StageAr
     if (g.nz == 1) return launch_rhs_flat_rows<CT, TIN, TST, true>(g, c, a, st);
   }
   if (c.roe) return launch_rhs_march<CT, TIN, TST, true>(g, c, a, st);
-  return launch_rhs_march<CT, TIN, TST, false>(g, c, a, st);
-
+  if constexpr (std::is_same<CT, double>::value) return launch_rhs_f64(g, c, a, st);
+  else return launch_rhs_march<CT, TIN, TST, false>(g, c, a, st);
 }
 
 template cudaError_t launch_rhs_stage<double, double, double>(const GridDesc&, const Coef<double>&,
