@@ -315,6 +315,28 @@ __device__ __forceinline__ double f2d(float f) {
   return __hiloint2double((int)(sign | hi), (int)lo);
 }
 
+// 1/x: the FP32 reciprocal y and y (1 + e + e^2), e = 1 - x y, which cubes its relative error
+// of 2^-22 (three FP64 instructions, the quotient takes some eight); the quotient itself
+// outside FP32's range.
+__device__ __forceinline__ double recip(double x) {
+  const float s = d2f(x), a = fabsf(s);
+  if (!(a > 1e-30f && a < 1e30f)) return 1.0 / x;
+  const double y = f2d(1.0f / s);
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// sqrt(x) in the same way: t = x y with y = rsqrt(x) of FP32, and t (1 + e/2 + 3 e^2/8),
+// e = 1 - t y
+__device__ __forceinline__ double root(double x) {
+  const float s = d2f(x);
+  if (!(s > 1e-30f && s < 1e30f)) return sqrt(x);
+  const double y = f2d(rsqrtf(s));
+  const double t = x * y;
+  const double e = fma(-t, y, 1.0);
+  return fma(t * e, fma(0.375, e, 0.5), t);
+}
+
 // conversions used by the templated kernels: to the compute type / back to FP64
 template <class T> __device__ __forceinline__ T cvt(double x);
 template <> __device__ __forceinline__ double cvt<double>(double x) { return x; }

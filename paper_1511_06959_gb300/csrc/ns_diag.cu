@@ -419,6 +419,146 @@ __device__ T sigma1_of(const T M[5][5]) {
   return sqrt(l > T(0) ? l : T(0));
 }
 
+// The same in FP64.  Reduction and iteration above are some 400 FP64 instructions of a cell
+// (GB300 issues FP64 at 1/64 of the FP32 rate), so the eigenvector is found in FP32 and only
+// the eigenvalue in FP64.  B = M^T M is squared, at unit trace, until it is v v^T (its trace
+// before the next squaring, sum(lambda^2) / sum(lambda)^2, tells); then, for any unit v,
+//   lambda = rho + r^T (lambda - B')^-1 r,  rho = v^T B v, r = B v - rho v, B' = B off v,
+// exactly.  rho and r are taken in FP64 from M; the second term, some 1e-14 of the first, in
+// FP32 with rho for lambda (a third-order change), as r^T (rho - B + v v^T)^-1 r by LDL^T.
+// Its own error is the FP32 roundings (5e-7) over the relative gap g to the next eigenvalue,
+// which 1 / g ~ rel rho / |r|^2 measures: where that would pass 3e-16 (g below about 1e-2),
+// where the squaring has not settled, and for matrices outside FP32's squares, the general
+// iteration takes over.  128x64x64 cells: k_sigma1 in FP64 took 898 us with the general
+// iteration in every cell, 707 us with it started from the FP32 eigenvalue, and 300 us so,
+// with the reciprocals and roots by recip() and root() and the folded entries of M.
+struct Mat5 {
+  double m[5][5];
+};
+__device__ __noinline__ double sigma1_general(Mat5 A) { return sigma1_of<double, 5>(A.m); }
+
+__device__ __forceinline__ double sigma1_f64(const double (&M)[5][5]) {
+  float F[5][5], mx = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 5; ++i)
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      F[i][j] = d2f(M[i][j]);
+      mx = fmaxf(mx, fabsf(F[i][j]));
+    }
+  const float is = 1.0f / mx;
+  float B[5][5], P[5][5], tr = 0.0f;   // lower triangles
+#pragma unroll
+  for (int i = 0; i < 5; ++i)
+#pragma unroll
+    for (int j = 0; j < 5; ++j) F[i][j] *= is;
+#pragma unroll
+  for (int i = 0; i < 5; ++i)
+#pragma unroll
+    for (int j = 0; j <= i; ++j) {
+      float a = 0.0f;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) a = fmaf(F[k][i], F[k][j], a);
+      B[i][j] = a;
+      if (i == j) tr += a;
+    }
+  const float it = 1.0f / tr;
+#pragma unroll
+  for (int i = 0; i < 5; ++i)
+#pragma unroll
+    for (int j = 0; j <= i; ++j) P[i][j] = B[i][j] * it;
+  bool ok = false;
+#pragma unroll 1
+  for (int n = 0; n < 10 && !ok; ++n) {
+    float Q[5][5], t = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+      for (int j = 0; j <= i; ++j) {
+        float a = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) a = fmaf(i > k ? P[i][k] : P[k][i], j > k ? P[j][k] : P[k][j], a);
+        Q[i][j] = a;
+        if (i == j) t += a;
+      }
+    ok = t > 0.9999f;
+    const float q = 1.0f / t;
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+      for (int j = 0; j <= i; ++j) P[i][j] = Q[i][j] * q;
+  }
+  // v: the column of v v^T with the largest diagonal entry
+  float v[5], vm = P[0][0];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) v[i] = P[i][0];
+#pragma unroll
+  for (int j = 1; j < 5; ++j) {
+    const bool up = P[j][j] > vm;
+    vm = up ? P[j][j] : vm;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) v[i] = up ? (i > j ? P[i][j] : P[j][i]) : v[i];
+  }
+  const float iv = rsqrtf(vm);
+  double vd[5], vv = 0.0, yy = 0.0, y[5], r[5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    v[i] *= iv;
+    vd[i] = f2d(v[i]);
+    vv = fma(vd[i], vd[i], vv);
+  }
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    double a = 0.0;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) a = fma(M[i][j], vd[j], a);
+    y[i] = a;
+    yy = fma(a, a, yy);
+  }
+  const double rho = yy * recip(vv);
+  const float is2 = is * is;
+  const float rf = d2f(rho) * is2;
+  float rr = 0.0f, x[5];
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    double a = -rho * vd[j];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) a = fma(M[i][j], y[i], a);
+    r[j] = a;
+    x[j] = d2f(r[j]) * is2;
+    rr = fmaf(x[j], x[j], rr);
+  }
+  // x^T K^-1 x, K = rf I - B + rf v v^T
+  float K[5][5], del = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 5; ++i)
+#pragma unroll
+    for (int j = 0; j <= i; ++j) K[i][j] = fmaf(rf * v[i], v[j], (i == j ? rf : 0.0f) - B[i][j]);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    ok = ok && K[k][k] > 0.0f;
+    const float id = 1.0f / K[k][k];
+    del = fmaf(x[k] * x[k], id, del);
+#pragma unroll
+    for (int i = k + 1; i < 5; ++i) {
+      const float l = K[i][k] * id;
+      x[i] = fmaf(-l, x[k], x[i]);
+#pragma unroll
+      for (int j = k + 1; j <= i; ++j) K[i][j] = fmaf(-l, K[j][k], K[i][j]);
+    }
+  }
+  ok = ok && mx > 1e-14f && mx < 1e14f && del * del <= 6e-10f * rr;
+  if (!ok) {
+    Mat5 A;
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+      for (int j = 0; j < 5; ++j) A.m[i][j] = M[i][j];
+    return sigma1_general(A);
+  }
+  return root(fma(rho, f2d(del / rf), rho));
+}
+
 // Growth matrix M = M1 - M2 of one cell from central differences of rho, u, p, a, b at
 // its six neighbours (closed forms of section "Energy analysis").
 template <class CT>
@@ -473,6 +613,12 @@ __device__ __forceinline__ void growth_matrix(const GridDesc& g, const Coef<CT>&
   M[4][4] -= gm1 / CT(2) * div;
 }
 
+// a / b: the quotient in FP32, a times the Newton reciprocal in FP64; the square root
+__device__ __forceinline__ float quot(float a, float b) { return a / b; }
+__device__ __forceinline__ double quot(double a, double b) { return a * recip(b); }
+__device__ __forceinline__ float sqroot(float a) { return sqrt(a); }
+__device__ __forceinline__ double sqroot(double a) { return root(a); }
+
 // sigma_1 by plane marching.  A CTA owns a TX x SG_TY tile of columns and a range of
 // planes (march_range, as the stencil kernels); the primitives (rho, u1, u2, u3, p, a, b)
 // of three consecutive planes of the tile and its one-cell halo sit in a shared-memory
@@ -520,6 +666,9 @@ __global__ void __launch_bounds__(sgk::NT, sizeof(CT) == 4 ? 4 : 1) k_sigma1(Gri
   const size_t boxoff = (size_t)b * 5 * g.cells;
   const CT gam = c.gamma, gm1 = c.gm1;
   const CT fb = CT(1) / sqrt(gam), fa = sqrt(gm1 / gam);
+  // FP64: the factors of the differences of c and of the divergence
+  [[maybe_unused]] const CT fb2 = CT(0.5) * fb, fa2 = CT(0.5) * fa, fa4 = fa2 - CT(2) * fa / gm1,
+                            f04 = CT(-0.5) * sqrt(gm1), f44 = CT(0.5) - CT(0.5) * gm1;
   int ho[2];
 #pragma unroll
   for (int it = 0; it < 2; ++it) {
@@ -544,17 +693,21 @@ __global__ void __launch_bounds__(sgk::NT, sizeof(CT) == 4 ? 4 : 1) k_sigma1(Gri
       if (t < SP) {
         // the operations of prim_at()
         const CT rho = q[it][0];
-        const CT ir = CT(1) / rho;
+        const CT ir = quot(CT(1), rho);
         const CT u0 = q[it][1] * ir, u1 = q[it][2] * ir, u2 = q[it][3] * ir;
         const CT p = (gam - CT(1)) * (q[it][4] - CT(0.5) * rho * (u0 * u0 + u1 * u1 + u2 * u2));
-        const CT cs = sqrt(gam * p * ir);
+        const CT cs = sqroot(gam * p * ir);
         P[0 * SP + t] = rho;
         P[1 * SP + t] = u0;
         P[2 * SP + t] = u1;
         P[3 * SP + t] = u2;
         P[4 * SP + t] = p;
-        P[5 * SP + t] = fa * cs;
-        P[6 * SP + t] = fb * cs;
+        if constexpr (sizeof(CT) == 8) {
+          P[5 * SP + t] = cs;   // a = fa c and b = fb c enter through the factors of the differences
+        } else {
+          P[5 * SP + t] = fa * cs;
+          P[6 * SP + t] = fb * cs;
+        }
       }
     }
   };
@@ -594,48 +747,92 @@ __global__ void __launch_bounds__(sgk::NT, sizeof(CT) == 4 ? 4 : 1) k_sigma1(Gri
           pl = Pp[v * SP + ic];
         }
       };
-      CT drho[3], du[3][3], dp[3], da[3], db[3];
+      CT M[5][5], s1;
+      if constexpr (sizeof(CT) == 8) {
+        // the entries of growth_matrix() with the constant factors folded
+        const CT rho0 = P0[0 * SP + ic], c0 = P0[5 * SP + ic];
+        const CT q0 = quot(CT(1), rho0 * c0);
+        const CT kb = fb * c0 * c0 * q0;         // b / rho
+        const CT kp = CT(0.5) * fa * gam * q0;   // a / (2 p)
+        CT du[3][3], drho[3], dp[3], dc[3];
 #pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const CT h = c.hidx[j];
-        CT m, pl;
-        nb(0, j, m, pl);
-        drho[j] = (pl - m) * h;
-        nb(4, j, m, pl);
-        dp[j] = (pl - m) * h;
-        nb(5, j, m, pl);
-        da[j] = (pl - m) * h;
-        nb(6, j, m, pl);
-        db[j] = (pl - m) * h;
+        for (int j = 0; j < 3; ++j) {
+          CT m, pl;
+          nb(0, j, m, pl);
+          drho[j] = (pl - m) * c.hidx[j];
+          nb(4, j, m, pl);
+          dp[j] = (pl - m) * c.hidx[j];
+          nb(5, j, m, pl);
+          dc[j] = (pl - m) * c.hidx[j];
 #pragma unroll
-        for (int kk = 0; kk < 3; ++kk) {
-          nb(1 + kk, j, m, pl);
-          du[kk][j] = (pl - m) * h;
+          for (int kk = 0; kk < 3; ++kk) {
+            nb(1 + kk, j, m, pl);
+            du[kk][j] = (pl - m) * c.hidx[j];
+          }
         }
+        const CT div = du[0][0] + du[1][1] + du[2][2], hd = CT(0.5) * div;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          M[1 + j][0] = fb2 * dc[j];
+          M[0][1 + j] = M[1 + j][0] - kb * drho[j];
+          M[4][1 + j] = fa4 * dc[j];
+          M[1 + j][4] = fa2 * dc[j] - kp * dp[j];
+#pragma unroll
+          for (int kk = 0; kk < 3; ++kk) M[1 + kk][1 + j] = kk == j ? hd - du[kk][j] : -du[kk][j];
+        }
+        M[0][0] = hd;
+        M[4][0] = CT(0);
+        M[0][4] = f04 * div;
+        M[4][4] = f44 * div;
+        if (g.nz == 1) {
+          // the (rho, u1, u2, p) block; the rest adds a zero eigenvalue
+#pragma unroll
+          for (int j = 0; j < 5; ++j) M[3][j] = M[j][3] = CT(0);
+        }
+        s1 = sigma1_f64(M);
+      } else {
+        CT drho[3], du[3][3], dp[3], da[3], db[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const CT h = c.hidx[j];
+          CT m, pl;
+          nb(0, j, m, pl);
+          drho[j] = (pl - m) * h;
+          nb(4, j, m, pl);
+          dp[j] = (pl - m) * h;
+          nb(5, j, m, pl);
+          da[j] = (pl - m) * h;
+          nb(6, j, m, pl);
+          db[j] = (pl - m) * h;
+#pragma unroll
+          for (int kk = 0; kk < 3; ++kk) {
+            nb(1 + kk, j, m, pl);
+            du[kk][j] = (pl - m) * h;
+          }
+        }
+        const CT rho0 = P0[0 * SP + ic], p0 = P0[4 * SP + ic], a0 = P0[5 * SP + ic], b0 = P0[6 * SP + ic];
+        const CT div = du[0][0] + du[1][1] + du[2][2];
+#pragma unroll
+        for (int i2 = 0; i2 < 5; ++i2)
+#pragma unroll
+          for (int j2 = 0; j2 < 5; ++j2) M[i2][j2] = i2 == j2 ? CT(0.5) * div : CT(0);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          M[0][1 + j] = M[1 + j][0] = CT(0.5) * db[j];
+          M[1 + j][4] = M[4][1 + j] = CT(0.5) * da[j];
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          M[0][1 + j] -= b0 / rho0 * drho[j];
+#pragma unroll
+          for (int kk = 0; kk < 3; ++kk) M[1 + kk][1 + j] -= du[kk][j];
+          M[4][1 + j] -= CT(2) / gm1 * da[j];
+          M[1 + j][4] -= a0 / (CT(2) * p0) * dp[j];
+        }
+        M[0][4] -= sqrt(gm1) / CT(2) * div;
+        M[4][4] -= gm1 / CT(2) * div;
+        s1 = g.nz == 1 ? sigma1_of<CT, 4>(M) : sigma1_of<CT, 5>(M);
       }
-      const CT rho0 = P0[0 * SP + ic], p0 = P0[4 * SP + ic], a0 = P0[5 * SP + ic], b0 = P0[6 * SP + ic];
-      CT M[5][5];
-      const CT div = du[0][0] + du[1][1] + du[2][2];
-#pragma unroll
-      for (int i2 = 0; i2 < 5; ++i2)
-#pragma unroll
-        for (int j2 = 0; j2 < 5; ++j2) M[i2][j2] = i2 == j2 ? CT(0.5) * div : CT(0);
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        M[0][1 + j] = M[1 + j][0] = CT(0.5) * db[j];
-        M[1 + j][4] = M[4][1 + j] = CT(0.5) * da[j];
-      }
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        M[0][1 + j] -= b0 / rho0 * drho[j];
-#pragma unroll
-        for (int kk = 0; kk < 3; ++kk) M[1 + kk][1 + j] -= du[kk][j];
-        M[4][1 + j] -= CT(2) / gm1 * da[j];
-        M[1 + j][4] -= a0 / (CT(2) * p0) * dp[j];
-      }
-      M[0][4] -= sqrt(gm1) / CT(2) * div;
-      M[4][4] -= gm1 / CT(2) * div;
-      const CT s1 = g.nz == 1 ? sigma1_of<CT, 4>(M) : sigma1_of<CT, 5>(M);
       const size_t o = (size_t)b * g.cells + (size_t)k * g.plane + cp;
       if (sigd) {
         // FP64 contexts: sigma_1 and the rule's viscosity kept in FP64
@@ -855,11 +1052,36 @@ __device__ __forceinline__ T energy_cell(const TIN* __restrict__ w, const TIN* _
   return v0 * v0 + y1 * y1 + y2 * y2 + y3 * y3 + v4 * v4;
 }
 
+// The same in FP64 with its constants from the host, one reciprocal of r, one square root
+// (m = r c = sqrt(gamma r p)) and one reciprocal of m.  The kernel is bound by its FP64
+// operations: with the constants and the block reduction in every thread of RGS blocks, fewer
+// than two cells each, and quotients, it took 102 us of 128x64x64 cells, against 52 us.
+struct EnergyConst {
+  double gamma, gm1, igm1, sg, isg, sgg;   // gamma, gamma - 1, 1 / gm1, sqrt(gamma), 1 / sg, sqrt(gm1 / gamma)
+};
+__device__ __forceinline__ double energy_cell_f64(const double* __restrict__ w, const double* __restrict__ lam,
+                                                  size_t box, long long cells, long long i, const EnergyConst& c) {
+  const double* W = w + box + i;
+  const double* L = lam + box + i;
+  const double r = W[0], m1 = W[cells], m2 = W[2 * cells], m3 = W[3 * cells], e = W[4 * cells];
+  const double l0 = L[0], l1 = L[cells], l2 = L[2 * cells], l3 = L[3 * cells], l4 = L[4 * cells];
+  const double ir = recip(r);
+  const double u0 = m1 * ir, u1 = m2 * ir, u2 = m3 * ir;
+  const double k = 0.5 * (u0 * u0 + u1 * u1 + u2 * u2);
+  const double p = c.gm1 * (e - r * k);
+  const double m = root(c.gamma * r * p);
+  const double y0 = l0 + u0 * l1 + u1 * l2 + u2 * l3 + k * l4;
+  const double y1 = l1 + u0 * l4, y2 = l2 + u1 * l4, y3 = l3 + u2 * l4;
+  const double y4 = m * c.igm1 * l4;
+  const double v0 = c.sg * r * r * recip(m) * y0 + c.isg * y4;
+  const double v4 = c.sgg * y4;
+  return v0 * v0 + r * r * (y1 * y1 + y2 * y2 + y3 * y3) + v4 * v4;
+}
 
 // E[b] = dV sum_cells |v_hat|^2; the last block of each box adds the block partials in
 // fixed order (ticket: per-box counters, zero on entry and on exit).
 template <class T, class TIN>
-__global__ void __launch_bounds__(RB, sizeof(T) == 4 ? 8 : 1) k_energy(GridDesc g, double gamma, double dV, const TIN* __restrict__ w,
+__global__ void __launch_bounds__(RB, sizeof(T) == 4 ? 8 : 1) k_energy(GridDesc g, EnergyConst c, double dV, const TIN* __restrict__ w,
                                                const TIN* __restrict__ lam, double* partial, double* E,
                                                unsigned* err, unsigned* ticket) {
   pdl_enter();
@@ -874,7 +1096,7 @@ __global__ void __launch_bounds__(RB, sizeof(T) == 4 ? 8 : 1) k_energy(GridDesc 
     // per warp, the warps' values added in order by thread 0
     float hi = 0.0f, lo = 0.0f;
     for (long long i = (long long)blockIdx.x * RB + threadIdx.x; i < g.cells; i += (long long)gridDim.x * RB)
-      df_add(hi, lo, energy_cell<T, TIN>(w, lam, box, g.cells, i, T(gamma)), 0.0f);
+      df_add(hi, lo, energy_cell<T, TIN>(w, lam, box, g.cells, i, T(c.gamma)), 0.0f);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
       df_add(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
@@ -885,7 +1107,7 @@ __global__ void __launch_bounds__(RB, sizeof(T) == 4 ? 8 : 1) k_energy(GridDesc 
     __syncthreads();   // sh is reused by the last block's reduction
   } else {
     for (long long i = (long long)blockIdx.x * RB + threadIdx.x; i < g.cells; i += (long long)gridDim.x * RB)
-      acc += energy_cell<T, TIN>(w, lam, box, g.cells, i, T(gamma));
+      acc += energy_cell_f64(w, lam, box, g.cells, i, c);
     acc = block_reduce(acc, sh, AddOp());
   }
   double* pb = partial + (size_t)b * gridDim.x;
@@ -1161,14 +1383,21 @@ cudaError_t launch_visc_apply(const GridDesc& g, const double* idx2, const doubl
   return launch_pdl(k_visc_apply, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, g, idx2[0], idx2[1], idx2[2], split[0], split[1], split[2], nu, a, out);
 }
 
+static EnergyConst energy_const(double gamma) {
+  const double gm1 = gamma - 1.0, sg = sqrt(gamma);
+  return {gamma, gm1, 1.0 / gm1, sg, 1.0 / sg, sqrt(gm1 / gamma)};
+}
+
 cudaError_t launch_energy(const GridDesc& g, double gamma, double dV, const double* w, const double* lam,
                           double* E, double* scratch, unsigned* err, bool fp32_transform, unsigned* ticket,
                           cudaStream_t st) {
-  dim3 grid(RGS, g.batch);
+  // FP64: four blocks a SM, as many as are resident, so that a thread has several cells
+  dim3 grid(fp32_transform ? RGS : 608, g.batch);
+  const EnergyConst c = energy_const(gamma);
   cudaError_t e = fp32_transform
-                      ? launch_pdl(k_energy<float, double>, grid, dim3(RB), 0, st, g, gamma, dV, w, lam, scratch, E,
+                      ? launch_pdl(k_energy<float, double>, grid, dim3(RB), 0, st, g, c, dV, w, lam, scratch, E,
                                    err, ticket)
-                      : launch_pdl(k_energy<double, double>, grid, dim3(RB), 0, st, g, gamma, dV, w, lam, scratch,
+                      : launch_pdl(k_energy<double, double>, grid, dim3(RB), 0, st, g, c, dV, w, lam, scratch,
                                    E, err, ticket);
   count_launch();
   return e;
@@ -1177,7 +1406,7 @@ cudaError_t launch_energy(const GridDesc& g, double gamma, double dV, const doub
 cudaError_t launch_energy_mirrors(const GridDesc& g, double gamma, double dV, const float* wf, const float* lamf,
                                   double* E, double* scratch, unsigned* err, unsigned* ticket, cudaStream_t st) {
   dim3 grid(RGS, g.batch);
-  cudaError_t e = launch_pdl(k_energy<float, float>, grid, dim3(RB), 0, st, g, gamma, dV, wf, lamf, scratch, E, err,
+  cudaError_t e = launch_pdl(k_energy<float, float>, grid, dim3(RB), 0, st, g, energy_const(gamma), dV, wf, lamf, scratch, E, err,
                              ticket);
   count_launch();
   return e;

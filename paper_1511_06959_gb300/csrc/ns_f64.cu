@@ -111,17 +111,6 @@ Consts consts_of(const Coef<double>& c) {
 // the place, nor the result on how the planes are cut into pieces.
 __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
 
-// 1/x: the FP32 reciprocal and two Newton steps y += y (1 - x y), which square its relative
-// error of 2^-23 twice (four FP64 instructions, the quotient takes twice as many); the
-// quotient itself outside FP32's range.
-__device__ __forceinline__ double recip(double x) {
-  const float s = fabsf(d2f(x));
-  if (!(s > 1e-30f && s < 1e30f)) return 1.0 / x;
-  double y = f2d(1.0f / d2f(x));
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
-}
-
 // x-face terms of shared position i (own row): a1 = d u_x / dy, a2 = d u_x / dz, d1 = the
 // divergence's y and z parts.  U0, Um, Up: velocity (stride SP) of planes k, k-1, k+1.
 __device__ __forceinline__ void x_terms(const Consts& K, const double* U0, const double* Um, const double* Up, int i,
