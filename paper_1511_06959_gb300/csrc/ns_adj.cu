@@ -521,12 +521,42 @@ __device__ __forceinline__ void add_viscosity(const Coef<CT>& c, const double nu
   }
 }
 
+// Operands of the epilogue that a run's outermost stages read: the FP64 adjoint and the
+// source sensitivities.  They are loaded ahead of the assembly: read where they are used,
+// each group waited for memory in turn, behind the stores before it.  A step's last stage of
+// 128x64x64 cells with a source was active for 130,000 cycles, the others for 74,000; the
+// step went from 243 to 219 us (Roe 526 to 467 us).  OUTER: the stages that have such
+// operands; the others are a variant without them, since their registers made those stages 2%
+// slower.
+template <class TST>
+struct EpiIn {
+  double lam[5], sbar[5];
+  TST SB[5];
+};
+template <bool OUTER, class TIN, class TA, class TST>
+__device__ __forceinline__ void epi_load(EpiIn<TST>& e, const GridDesc& g, const AdjArgs<TIN, TA, TST>& a, size_t pbase,
+                                         size_t fc, int cp, long long n5) {
+  if (OUTER && a.lam_out && a.lam_in) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) e.lam[v] = NS_LD(g, a.lam_in, pbase + v * fc, cp, n5);
+  }
+  if (a.SBin) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) e.SB[v] = NS_LD(g, a.SBin, pbase + v * fc, cp, n5);
+  }
+  if (OUTER && a.sbar) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) e.sbar[v] = NS_LD(g, a.sbar, pbase + v * fc, cp, n5);
+  }
+}
+
 // Epilogue of one cell (each optional operand tested once): see the file comment.
 // Ac: the cell's adjoint input, component stride astr.
-template <class CT, class TIN, class TA, class TST>
+template <bool OUTER, bool AHEAD, class CT, class TIN, class TA, class TST>
 __device__ __forceinline__ void adj_epilogue(const GridDesc& g, const AdjArgs<TIN, TA, TST>& a, int b, int k, int gx,
                                              int gy, size_t pbase, size_t fc, int cp, long long n5, const CT gin[5],
-                                             const CT lfv[5], const CT gout[5], const CT* Ac, int astr) {
+                                             const CT lfv[5], const EpiIn<TST>& ein, const CT gout[5], const CT* Ac,
+                                             int astr) {
   CT gs[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) gs[v] = gin[v] + gout[v];
@@ -534,13 +564,13 @@ __device__ __forceinline__ void adj_epilogue(const GridDesc& g, const AdjArgs<TI
 #pragma unroll
     for (int v = 0; v < 5; ++v) NS_ST(g, a.Gout, pbase + v * fc, cp, n5, gs[v]);
   }
-  if (a.lam_out) {
+  if (OUTER && a.lam_out) {
     double lv[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) lv[v] = widen(gs[v]);
     if (a.lam_in) {
 #pragma unroll
-      for (int v = 0; v < 5; ++v) lv[v] = NS_LD(g, a.lam_in, pbase + v * fc, cp, n5) + lv[v];
+      for (int v = 0; v < 5; ++v) lv[v] = (AHEAD ? ein.lam[v] : NS_LD(g, a.lam_in, pbase + v * fc, cp, n5)) + lv[v];
     }
     if (a.obj_ndsc && (gx == a.obj_iL || gx == a.obj_iR)) {
       // the objective source of this step on the plane's two columns, added after
@@ -566,22 +596,23 @@ __device__ __forceinline__ void adj_epilogue(const GridDesc& g, const AdjArgs<TI
     for (int v = 0; v < 5; ++v)
       NS_ST(g, a.Anext, pbase + v * fc, cp, n5, CT(a.cl) * lfv[v] + CT(a.cg) * gout[v] + CT(a.cs) * gs[v]);
   }
-  if (a.SBout || a.sbar) {
+  if (a.SBout || (OUTER && a.sbar)) {
     CT ss[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) ss[v] = Ac[v * astr];
     if (a.SBin) {
 #pragma unroll
-      for (int v = 0; v < 5; ++v) ss[v] = NS_LD(g, a.SBin, pbase + v * fc, cp, n5) + ss[v];
+      for (int v = 0; v < 5; ++v) ss[v] = (AHEAD ? ein.SB[v] : NS_LD(g, a.SBin, pbase + v * fc, cp, n5)) + ss[v];
     }
     if (a.SBout) {
 #pragma unroll
       for (int v = 0; v < 5; ++v) NS_ST(g, a.SBout, pbase + v * fc, cp, n5, ss[v]);
     }
-    if (a.sbar) {
+    if (OUTER && a.sbar) {
 #pragma unroll
       for (int v = 0; v < 5; ++v)
-        NS_ST(g, a.sbar, pbase + v * fc, cp, n5, NS_LD(g, a.sbar, pbase + v * fc, cp, n5) + widen(ss[v]));
+        NS_ST(g, a.sbar, pbase + v * fc, cp, n5,
+              (AHEAD ? ein.sbar[v] : NS_LD(g, a.sbar, pbase + v * fc, cp, n5)) + widen(ss[v]));
     }
   }
 }
@@ -589,7 +620,7 @@ __device__ __forceinline__ void adj_epilogue(const GridDesc& g, const AdjArgs<TI
 // values per face packet: 7 (viscous and face velocity), plus 10 with Roe dissipation
 template <bool ROE> constexpr int npk() { return ROE ? 17 : 7; }
 
-template <class CT, class TIN, class TA, class TST, bool ROE>
+template <class CT, class TIN, class TA, class TST, bool ROE, bool OUTER>
 __global__ void __launch_bounds__(NT, AdjMinBlocks<CT, ROE>::value) k_adj_stage(GridDesc g, Coef<CT> c, AdjArgs<TIN, TA, TST> a) {
   pdl_enter();
   constexpr int NPK = npk<ROE>();
@@ -719,6 +750,10 @@ __global__ void __launch_bounds__(NT, AdjMinBlocks<CT, ROE>::value) k_adj_stage(
     __syncthreads();
     if (more) adj_plane_store(pf, sQ + slot(k + 2) * 5 * SP, sA + slot(k + 2) * 5 * SP, sN + slot(k + 2) * SP,
                               with_nu);
+    // (the registers of the plane just stored)
+    EpiIn<TST> ein;
+    constexpr bool ahead = sizeof(CT) == 4;   // FP64 (Roe) has no registers left for them
+    if constexpr (ahead) if (valid) epi_load<OUTER>(ein, g, a, pbase, fc, cp, n5);
 
     CT own_p[3] = {CT(0), CT(0), CT(0)};
     if (valid) {
@@ -810,7 +845,7 @@ __global__ void __launch_bounds__(NT, AdjMinBlocks<CT, ROE>::value) k_adj_stage(
         add_viscosity<SP, true>(c, a.nus, A0, Ap, am, ic, N0[ic], N0[ic - 1], N0[ic + 1], N0[ic - SX], N0[ic + SX],
                                 nzm, sN[sp * SP + ic], gout);
       }
-      adj_epilogue(g, a, b, k, gx, gy, pbase, fc, cp, n5, gin, lfv, gout, A0 + ic, SP);
+      adj_epilogue<OUTER, ahead>(g, a, b, k, gx, gy, pbase, fc, cp, n5, gin, lfv, ein, gout, A0 + ic, SP);
     }
 #pragma unroll
     for (int v = 0; v < NPK; ++v) zlo[v] = zhi[v];
@@ -940,6 +975,27 @@ __global__ void __launch_bounds__(FlatTile<TYF>::NT) k_adj_flat(GridDesc g, Coef
 #pragma unroll
     for (int v = 0; v < NPK; ++v) sFY[(v * (TYF + 1) + fy) * TX + lane] = pk[v];
   }
+  // the epilogue's operands: on single-row tiles (the smallest boxes, where the length of the
+  // chain counts) in FP32 ahead of the barriers; elsewhere at their use, since the registers
+  // would cost resident CTAs (400x400: 68 us per adjoint step at their use, 83 us ahead)
+  constexpr bool ahead = sizeof(CT) == 4 && TYF == 1;
+  CT gin0[5] = {CT(0), CT(0), CT(0), CT(0), CT(0)};
+  CT lfv0[5] = {CT(0), CT(0), CT(0), CT(0), CT(0)};
+  EpiIn<TST> ein;
+  auto operands = [&](int cp, CT (&gin)[5], CT (&lfv)[5]) {
+    if (a.Gin) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) gin[v] = NS_LD(g, a.Gin, box + v * fc, cp, n5);
+    }
+    if (a.Anext) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) lfv[v] = NS_LD(g, a.lamf, box + v * fc, cp, n5);
+    }
+    if constexpr (ahead) epi_load<true>(ein, g, a, box, fc, cp, n5);
+  };
+  if constexpr (ahead) {
+    if (wid == 0 && x0 + lane < g.nx && y0 < g.ny) operands(y0 * g.nx + x0 + lane, gin0, lfv0);
+  }
   __syncthreads();
   // viscous part, component v of (u1, u2, u3, e) of row ty
   for (int job = wid; job < 4 * TYF; job += T::NW) {
@@ -970,16 +1026,13 @@ __global__ void __launch_bounds__(FlatTile<TYF>::NT) k_adj_flat(GridDesc g, Coef
     const int tx = lane, gx = x0 + tx, gy = y0 + ty;
     if (gx >= g.nx || gy >= g.ny) continue;
     const int ic = (ty + 1) * SX + tx + 1, cp = gy * g.nx + gx;
-    CT gin[5] = {CT(0), CT(0), CT(0), CT(0), CT(0)};
-    CT lfv[5] = {CT(0), CT(0), CT(0), CT(0), CT(0)};
-    if (a.Gin) {
+    CT gin[5], lfv[5];
 #pragma unroll
-      for (int v = 0; v < 5; ++v) gin[v] = NS_LD(g, a.Gin, box + v * fc, cp, n5);
+    for (int v = 0; v < 5; ++v) {
+      gin[v] = ahead ? gin0[v] : CT(0);
+      lfv[v] = ahead ? lfv0[v] : CT(0);
     }
-    if (a.Anext) {
-#pragma unroll
-      for (int v = 0; v < 5; ++v) lfv[v] = NS_LD(g, a.lamf, box + v * fc, cp, n5);
-    }
+    if constexpr (!ahead) operands(cp, gin, lfv);
     CT rs[5] = {CT(0), CT(0), CT(0), CT(0), CT(0)};
     if constexpr (ROE) {
       const int fl = ty * (TX + 1) + tx, yl = ty * TX + tx;
@@ -1008,7 +1061,7 @@ __global__ void __launch_bounds__(FlatTile<TYF>::NT) k_adj_flat(GridDesc g, Coef
       const CT nc = N[ic], nxm = N[ic - 1], nxp = N[ic + 1], nym = N[ic - SX], nyp = N[ic + SX];
       add_viscosity<SPT, false>(c, a.nus, A, A, static_cast<const CT*>(nullptr), ic, nc, nxm, nxp, nym, nyp, CT(0), CT(0), gout);
     }
-    adj_epilogue(g, a, b, 0, gx, gy, box, fc, cp, n5, gin, lfv, gout, A + ic, SPT);
+    adj_epilogue<true, ahead>(g, a, b, 0, gx, gy, box, fc, cp, n5, gin, lfv, ein, gout, A + ic, SPT);
   }
 }
 
@@ -1040,11 +1093,11 @@ static cudaError_t launch_adj_flat_rows(const GridDesc& g, const Coef<CT>& c, co
                            : launch_adj_flat<CT, TIN, TA, TST, ROE, 4>(g, c, a, st);
 }
 
-template <class CT, class TIN, class TA, class TST, bool ROE>
+template <class CT, class TIN, class TA, class TST, bool ROE, bool OUTER>
 static cudaError_t launch_adj_march(const GridDesc& g, const Coef<CT>& c, const AdjArgs<TIN, TA, TST>& a,
                                      cudaStream_t st) {
   const size_t smem = adj_smem_bytes<CT, ROE>();
-  auto kern = k_adj_stage<CT, TIN, TA, TST, ROE>;
+  auto kern = k_adj_stage<CT, TIN, TA, TST, ROE, OUTER>;
   static MarchShape<TX, TY> shape;
   int ctas = 0;
   GridDesc gm = g;
@@ -1066,9 +1119,10 @@ cudaError_t launch_adj_stage(const GridDesc& g, const Coef<CT>& c, const AdjArgs
   if constexpr (std::is_same<CT, double>::value) {
     if (g.nz == 1) return adjk::launch_adj_flat_rows<CT, TIN, TA, TST, true>(g, c, a, st);
   }
-  if (c.roe) return adjk::launch_adj_march<CT, TIN, TA, TST, true>(g, c, a, st);
+  if (c.roe) return adjk::launch_adj_march<CT, TIN, TA, TST, true, true>(g, c, a, st);
   if constexpr (std::is_same<CT, double>::value) return launch_adj_f64(g, c, a, st);
-  else return adjk::launch_adj_march<CT, TIN, TA, TST, false>(g, c, a, st);
+  else if (a.lam_out || a.sbar) return adjk::launch_adj_march<CT, TIN, TA, TST, false, true>(g, c, a, st);
+  else return adjk::launch_adj_march<CT, TIN, TA, TST, false, false>(g, c, a, st);
 }
 
 template cudaError_t launch_adj_stage<double, double, double, double>(

@@ -355,6 +355,18 @@ __global__ void __launch_bounds__(NT, RhsMinBlocks<CT, ROE>::value) k_rhs_stage(
     __syncthreads();
     // the epilogue reads only the face fluxes: plane k+2 replaces plane k-1 in the ring now
     if (more) plane_store(pf, sQ + sm * 5 * SP);
+    // the step's FP64 state, in the registers of the plane just stored, ahead of its use
+    // (with Roe's registers at its use: 104.4 us a step of 128x64x64 cells, 105.2 us ahead)
+    double e_wbase[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    auto load_wbase = [&]() {
+      if (a.wout && a.wbase) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) e_wbase[v] = NS_LD(g, a.wbase, pb + v * (size_t)g.cells, cp, n5);
+      }
+    };
+    if constexpr (!std::is_same<CT, Dual>::value && !ROE) {
+      if (valid) load_wbase();
+    }
     if (valid) {
       CT R[5];
 #pragma unroll
@@ -393,12 +405,8 @@ __global__ void __launch_bounds__(NT, RhsMinBlocks<CT, ROE>::value) k_rhs_stage(
           const CT inc = CT(a.cacc) * Rv[v];
           dv[v] = e_dacc[v] + inc;
         }
+        if constexpr (ROE) load_wbase();
         if (a.wout) {
-          double e_wbase[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-          if (a.wbase) {
-#pragma unroll
-            for (int v = 0; v < 5; ++v) e_wbase[v] = NS_LD(g, a.wbase, pb + v * (size_t)g.cells, cp, n5);
-          }
           if (a.wout_mirror) {
 #pragma unroll
             for (int v = 0; v < 5; ++v) {
@@ -460,6 +468,33 @@ __global__ void __launch_bounds__(FlatTile<TYF>::NT) k_rhs_flat(GridDesc g, Coef
   const size_t box = (size_t)b * 5 * g.cells;
   const long long n5 = 5 * g.cells * g.batch;   // field extent (debug bounds checks)
   (void)n5;
+  // The operands of the warp's (row, component) jobs: on single-row tiles (the smallest boxes,
+  // where the length of the chain counts) ahead of the faces; elsewhere at their use, since the
+  // registers would cost resident CTAs.  64x64 FP32, a step of four stages: 12.0 us at their
+  // use, 11.3 us ahead; 400x400: 33.2 and 34.1 us.
+  struct JobIn {
+    CT src, dacc, base;
+    double wbase;
+  };
+  auto job_load = [&](int job) {
+    JobIn e{CT(0), CT(0), CT(0), 0.0};
+    const int x = x0 + lane, y = y0 + job / 5;
+    if (job >= 5 * TYF || x >= g.nx || y >= g.ny) return e;
+    const int cp = y * g.nx + x;
+    const size_t pv = box + (job % 5) * (size_t)g.cells;
+    if (a.src) e.src = cvt<CT>(NS_LD(g, a.src, pv, cp, n5));
+    if (a.dacc && !a.dacc_init) e.dacc = CT(NS_LD(g, a.dacc, pv, cp, n5));
+    if (a.Wout) e.base = CT(NS_LD(g, a.base, pv, cp, n5));
+    if (a.wout && a.wbase) e.wbase = NS_LD(g, a.wbase, pv, cp, n5);
+    return e;
+  };
+  constexpr bool ahead = TYF == 1;
+  constexpr int NJ = ahead ? (5 * TYF + T::NW - 1) / T::NW : 1;
+  JobIn in[NJ];
+  if constexpr (ahead) {
+#pragma unroll
+    for (int q = 0; q < NJ; ++q) in[q] = job_load(wid + q * T::NW);
+  }
   for (int t = tid; t < SPT; t += T::NT) {
     const int ly = t / SX, lx = t - ly * SX;
     const int o = wrap(y0 + ly - 1, g.ny) * g.nx + wrap(x0 + lx - 1, g.nx);
@@ -510,25 +545,31 @@ __global__ void __launch_bounds__(FlatTile<TYF>::NT) k_rhs_flat(GridDesc g, Coef
     for (int v = 0; v < 5; ++v) sFY[(v * (TYF + 1) + fy) * TX + lane] = phi[v];
   }
   __syncthreads();
-  for (int job = wid; job < 5 * TYF; job += T::NW) {
+  auto job_done = [&](int job, const JobIn& e) {
     const int v = job % 5, ty = job / 5, tx = lane, x = x0 + tx, y = y0 + ty;
-    if (x >= g.nx || y >= g.ny) continue;
+    if (x >= g.nx || y >= g.ny) return;
     const int cp = y * g.nx + x;
     const size_t pv = box + v * (size_t)g.cells;
     const CT* fx = sFX + (v * TYF + ty) * (TX + 1) + tx;
     const CT* fy = sFY + (v * (TYF + 1) + ty) * TX + tx;
     CT R = -((fx[1] - fx[0]) * c.idx[0] + (fy[TX] - fy[0]) * c.idx[1]);
-    if (a.src) R = R + cvt<CT>(NS_LD(g, a.src, pv, cp, n5));
-    const CT dv = (a.dacc && !a.dacc_init ? CT(NS_LD(g, a.dacc, pv, cp, n5)) : CT(0)) + CT(a.cacc) * R;
+    if (a.src) R = R + e.src;
+    const CT dv = e.dacc + CT(a.cacc) * R;
     if (a.wout) {
-      const double wv = (a.wbase ? NS_LD(g, a.wbase, pv, cp, n5) : 0.0) + widen(dv);
+      const double wv = e.wbase + widen(dv);
       NS_ST(g, a.wout, pv, cp, n5, wv);
       if (a.wout_mirror) NS_ST(g, a.wout_mirror, pv, cp, n5, cvt<TST>(wv));
     } else if (a.dacc) {
       NS_ST(g, a.dacc, pv, cp, n5, dv);
     }
-    if (a.Wout)
-      NS_ST(g, a.Wout, pv, cp, n5, CT(NS_LD(g, a.base, pv, cp, n5)) + CT(a.cout) * R + CT(a.cd) * dv);
+    if (a.Wout) NS_ST(g, a.Wout, pv, cp, n5, e.base + CT(a.cout) * R + CT(a.cd) * dv);
+  };
+  if constexpr (ahead) {
+#pragma unroll
+    for (int q = 0; q < NJ; ++q)
+      if (wid + q * T::NW < 5 * TYF) job_done(wid + q * T::NW, in[q]);
+  } else {
+    for (int job = wid; job < 5 * TYF; job += T::NW) job_done(job, job_load(job));
   }
 }
 
