@@ -278,11 +278,11 @@ __device__ __forceinline__ void char_pullback(const double wc[5], int side, cons
 // those cells, packed so that all 32 lanes of a warp have one, and the other CTAs the
 // cells of whole rows, leaving out the packed ones.  With every cell in one grid, each
 // row's end cells held two of its three warps for the whole pull-back: 931 us per stage of
-// a 96x48x48 duct (a primal and an adjoint step: 4070 us, 511 us with this split and the Laplacian below).
+// a 96x48x48 duct (a primal and an adjoint step: 4070 us, 505 us with this split and the Laplacian below).
 struct EpiArgs {
   const double* gp;
   const double* A;
-  double sa, nus[3], i2[3];
+  double sa, snus[3], hi2[3];   // sa, sa nu factors (rho, rho u, rho E), 1 / (2 dx^2)
   int mode, first, last;
   const double* lam;
   double* G;
@@ -314,14 +314,14 @@ __device__ __forceinline__ void epilogue_cell(const GridDesc& g, const Pad& P, c
     const bool closed[6] = {P.ix && x == 0, P.ix && x == g.nx - 1, P.iy && y == 0, P.iy && y == g.ny - 1, false, false};
     double F[6];
 #pragma unroll
-    for (int d = 0; d < 6; ++d) F[d] = closed[d] ? 0.0 : (nc + widen(nb[q[d]])) * (0.5 * e.i2[d >> 1]);
+    for (int d = 0; d < 6; ++d) F[d] = closed[d] ? 0.0 : (nc + widen(nb[q[d]])) * e.hi2[d >> 1];
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
       const double* Ak = e.A + (long long)b * 5 * g.cells + (long long)k * g.cells;
       double L = 0.0;
 #pragma unroll
       for (int d = 0; d < 6; ++d) L += F[d] * (Ak[q[d]] - A[k]);
-      gc[k] += (sa * e.nus[k == 0 ? 0 : (k == 4 ? 2 : 1)]) * L;
+      gc[k] += e.snus[k == 0 ? 0 : (k == 4 ? 2 : 1)] * L;
     }
   }
   const long long op = (long long)b * 5 * P.cellsp + (long long)z * P.planep + (long long)(y + P.iy) * P.nxp + x + P.ix;
@@ -484,7 +484,7 @@ cudaError_t launch_bc_adj_epilogue(const GridDesc& g, const BcDesc& bc, const Bc
                                    const CT* W, const NU* nu, CT* seed, cudaStream_t st) {
   EpiArgs a;
   a.gp = gp; a.A = e.A; a.sa = e.sa;
-  for (int k = 0; k < 3; ++k) { a.nus[k] = e.nus[k]; a.i2[k] = e.i2[k]; }
+  for (int k = 0; k < 3; ++k) { a.snus[k] = e.sa * e.nus[k]; a.hi2[k] = 0.5 * e.i2[k]; }
   a.mode = e.mode; a.first = e.first; a.last = e.last;
   a.lam = e.lam; a.G = e.G; a.cl = e.cl; a.cg = e.cg; a.cs = e.cs;
   a.a_next = e.a_next; a.out = e.out; a.sbar = e.sbar;
