@@ -211,8 +211,14 @@ __device__ __forceinline__ const CT& yf(const CT* F, int j, int fy, int col) {
 // Face values of one plane slot, each face once.  Every thread computes its own cell's
 // lower x-face (shared row ty+1, fx = tx) and lower y-face (fy = ty, column tx+1); the
 // NRF remaining faces (x-faces of the halo rows and of the last column, y-faces of the
-// last row and of the halo columns) go to threads t < NRF.
+// last row and of the halo columns) go to NRF threads from T_RF on.
 constexpr int NRF = NF - 2 * NT;
+// First threads of the remaining faces and of the halo's z-faces.  A plane's barrier waits for
+// the warp with most of the tile's edges: warp 0 takes the last row of y-packets and warp 1 the
+// last column of x-packets, so the faces go to the last warps and the z-faces to those from
+// warp 2 on.  Adjoint step of 256x256x128 cells, all of them from thread 0 on: 2662 us, so:
+// 2615 us (128x64x64: 201.5 and 200.5 us).
+constexpr int T_RF = NT - (NRF + 31) / 32 * 32, T_H = NT >= 256 ? 2 * 32 : 0;
 static_assert(NRF == 2 * (SX - 1) + TY + SX + 2 * TY, "remaining faces of a plane slot");
 
 template <class CT>
@@ -239,8 +245,8 @@ __device__ __forceinline__ void fill_faces(CT* __restrict__ F, const CT* __restr
     face_s<1>(c, Q, A, iL, Q, A, iL + SX, sv, fb4);
     store_face(F, NXF + iL, sv, fb4);
   }
-  const int t = threadIdx.x;
-  if (t < NRF) {
+  const int t = (int)threadIdx.x - T_RF;
+  if (t >= 0 && t < NRF) {
     if (t < 2 * (SX - 1) + TY) {
       // x-faces: halo row 0, halo row SY-1, then the last face (fx = SX-2) of rows 1..TY
       int row, fx;
@@ -370,9 +376,9 @@ __device__ __forceinline__ void roe_packet(const Coef<CT>& c, const CT* QL, cons
 // z-face s-vectors between plane slots sL and sR at every shared column: the thread's own
 // column ic (its s-vector and Fb[4] also returned for its z-packet) and the NH halo
 // positions of the slot (rows 0 and SY-1, then columns 0 and SX-1 of rows 1..TY) by
-// threads t < NH.
+// NH threads from T_H on.
 constexpr int NH = 2 * SX + 2 * TY;
-static_assert(NH + NT == SP, "halo positions of a plane slot");
+static_assert(NH + NT == SP && T_H + NH <= NT && T_RF >= 0, "halo positions of a plane slot");
 
 template <class CT>
 __device__ __forceinline__ void fill_Z(CT* __restrict__ Z, const CT* __restrict__ sQ,
@@ -385,8 +391,8 @@ __device__ __forceinline__ void fill_Z(CT* __restrict__ Z, const CT* __restrict_
   face_s<2>(c, QL, AL, ic, QR, AR, ic, s_own, fb_own);
 #pragma unroll
   for (int j = 0; j < 3; ++j) Z[j * SP + ic] = s_own[j];
-  const int t = threadIdx.x;
-  if (t < NH) {
+  const int t = (int)threadIdx.x - T_H;
+  if (t >= 0 && t < NH) {
     int i;
     if (t < SX) i = t;
     else if (t < 2 * SX) i = (SY - 1) * SX + (t - SX);
