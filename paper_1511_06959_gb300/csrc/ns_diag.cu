@@ -625,7 +625,8 @@ __device__ __forceinline__ double sqroot(double a) { return root(a); }
 // ring, filled from register-staged loads one plane ahead, so each state is loaded and
 // converted once per CTA instead of seven times per cell.  The growth matrix of a cell
 // is then the closed form of growth_matrix() on those values (the same operations, so the
-// same sigma_1 bits).  Statistics: every CTA writes its (max, sum) for its box and zeros
+// same sigma_1 bits; in FP64 the ring holds the sound speed in place of a and b, and the
+// constant factors are folded).  Statistics: every CTA writes its (max, sum) for its box and zeros
 // for the other boxes; the last CTA (ticket[0]) reduces them per box in a fixed order.
 namespace sgk {
 constexpr int TY = 8;

@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(RB) k_box_means_final(int nblk, double inv_cel
 // rho u of three planes with a one-cell halo in a shared-memory ring, so each cell's state is loaded
 // and divided once per tile instead of seven times; a warp's 32 x 16 features go out
 // through shared memory as whole lines.  1.77 M cells in eight boxes: 115 us with a thread
-// per cell reading its six neighbours, 44 us now (27 us at the memory's rate).
+// per cell reading its six neighbours, 42 us now (27 us at the memory's rate).
 namespace fk {
 constexpr int FY = 8;
 constexpr int NT = TX * FY;

@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(NT, RhsMinBlocks<CT, ROE>::value) k_rhs_stage(
 // (row, component) of cells per warp.  Small boxes are bound by the length of this chain
 // and the number of SMs at work: 64x64 had 16 CTAs with the marching kernel.  One step of
 // four stages, marching kernel before, this one now: 64x64 FP64 136 and 23 us, FP32 21 and
-// 14 us; 400x400 FP64 659 and 307 us, FP32 46 and 35 us.
+// 11 us; 400x400 FP64 659 and 307 us, FP32 46 and 33 us.
 // ---------------------------------------------------------------------------------
 template <int TYF>
 struct FlatTile {
