@@ -227,8 +227,9 @@ int ns_max_wave_speed(ns_ctx* ctx, const double* w, double* out);
  * primal states to keep (ns_plan) and executes the plan on the context's stream
  * (ns_adjoint_run).  Schedules:
  *   NS_CKPT_ALL     keep every state, and on a periodic box every step's stage states when
- *                   they take at most 16 GiB (no recomputation; without them, and after
- *                   ns_set_pipeline(ctx, 0), each adjoint step recomputes its stages)
+ *                   they take at most 16 GiB and verify is off (no recomputation; without
+ *                   them, and after ns_set_pipeline(ctx, 0), each adjoint step
+ *                   recomputes its stages)
  *   NS_CKPT_STRIDE  keep every param-th state; replay one segment at a time and keep
  *                   all its states during its reversal.  The last segment is not
  *                   replayed: the forward pass keeps its states, so a sweep advances

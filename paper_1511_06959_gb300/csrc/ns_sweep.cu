@@ -364,11 +364,13 @@ bool pipelined(const ns_ctx* c, int nsteps, int schedule, int param, bool verify
 // boxes, 20 steps with gradients: 24.5 ms without, 19.1 ms with).  It does so while they
 // take at most KEEP_ALL_MAX bytes (about a sixteenth of the device's 280 GB) and unless
 // the caller asked for the smallest footprint (ns_set_pipeline(ctx, 0), NS_PIPELINE=0).
+// Not with snapshot checksums: those cover the snapshots alone, so a verified adjoint step
+// forms its mirror and its stages from the snapshot that has just passed.
 constexpr size_t KEEP_ALL_MAX = (size_t)16 << 30;
 
-bool keeps_all_stages(const ns_ctx* c, int nsteps, int schedule) {
+bool keeps_all_stages(const ns_ctx* c, int nsteps, int schedule, bool verify) {
   const bool on = c->pipeline < 0 ? pipeline_enabled() : c->pipeline != 0;
-  return on && schedule == NS_CKPT_ALL && !c->bounded() &&
+  return on && schedule == NS_CKPT_ALL && !c->bounded() && !verify &&
          (size_t)nsteps <= KEEP_ALL_MAX / 4 / align256(ns_i_stage_bytes(c));
 }
 
@@ -430,7 +432,7 @@ size_t ns_run_arena_bytes(const ns_ctx* c, const ns_run_opts* o) {
   if (make_plan(o->nsteps, o->schedule, o->param, P)) return 0;
   return layout_for(c, P.maxlive, o->mlp != nullptr, o->schedule, o->param, P.maxhost, o->verify != 0,
                     pipelined(c, o->nsteps, o->schedule, o->param, o->verify != 0),
-                    keeps_all_stages(c, o->nsteps, o->schedule) ? o->nsteps : 0)
+                    keeps_all_stages(c, o->nsteps, o->schedule, o->verify != 0) ? o->nsteps : 0)
       .total;
 }
 
@@ -898,7 +900,7 @@ static int forward_run_impl(ns_ctx* c, const double* w0, const double* s, const 
   }
   S->pipe = pipelined(c, o->nsteps, o->schedule, o->param, o->verify != 0);
   S->L = layout_for(c, S->P.maxlive, o->mlp != nullptr, o->schedule, o->param, S->P.maxhost, o->verify != 0,
-                    S->pipe, keeps_all_stages(c, o->nsteps, o->schedule) ? o->nsteps : 0);
+                    S->pipe, keeps_all_stages(c, o->nsteps, o->schedule, o->verify != 0) ? o->nsteps : 0);
   if (arena_bytes < S->L.total) {
     delete S;
     return NS_ERR_BUDGET;
