@@ -338,8 +338,11 @@ typedef struct {
 /* Device bytes the caller must provide as the arena of ns_adjoint_run (state slots,
  * two working states, one adjoint field, sigma_1 and nu fields, scalars; for a stride
  * plan one segment's kept stage states and mirrors, for a store-all plan every step's while
- * they take at most 16 GiB, and when the sweep is pipelined a
- * second set of them with param - 1 segment states per set, see ns_set_pipeline). */
+ * they take at most 16 GiB and verify is off, and when the sweep is pipelined a second set
+ * of them with param - 1 segment states per set, see ns_set_pipeline).  A store-all sweep
+ * also runs in an arena of the size without its kept stages (the answer after
+ * ns_set_pipeline(ctx, 0)) or more, recomputing them, with the same bits; an arena that
+ * misses the full size by less than one step's stages is NS_ERR_BUDGET all the same. */
 size_t ns_run_arena_bytes(const ns_ctx* ctx, const ns_run_opts* o);
 
 /* Host bytes of the snapshot arena of an NS_CKPT_STRIDE_HOST or NS_CKPT_REVOLVE_HOST sweep

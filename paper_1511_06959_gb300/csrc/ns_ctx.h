@@ -100,6 +100,8 @@ int ns_i_sigma1(ns_ctx* c, const double* w, const void* w_mirror, float* sigma1,
 // FP64 contexts: sigma_1 (and with nu != null the rule's viscosity) kept in FP64
 int ns_i_sigma1_f64(ns_ctx* c, const double* w, double* sigma1, double* stats, double lambda, double tau,
                     double* nu);
+// whether a sweep of these options runs in an arena of `bytes` (ns_run_arena_bytes)
+bool ns_i_arena_fits(const ns_ctx* c, const ns_run_opts* o, size_t bytes);
 size_t ns_i_stage_bytes(const ns_ctx* c);
 
 namespace ns {

@@ -102,7 +102,7 @@ int ns_estimate_lambda(ns_ctx* c, const double* w0, const double* s, const ns_ru
     if (!(lambdas[i] >= 0.0) || (i > 0 && !(lambdas[i] > lambdas[i - 1]))) return NS_ERR_ARG;
   const WorkLayout L = work_layout(c, o->nsteps);
   if (work_bytes < L.total) return NS_ERR_BUDGET;
-  if (arena_bytes < ns_run_arena_bytes(c, o)) return NS_ERR_BUDGET;
+  if (!ns_i_arena_fits(c, o, arena_bytes)) return NS_ERR_BUDGET;
   char* q = (char*)work;
   double* lam0 = (double*)q;
   double* sb[2] = {(double*)(q + L.field), (double*)(q + 2 * L.field)};

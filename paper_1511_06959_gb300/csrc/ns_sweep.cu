@@ -407,7 +407,29 @@ Layout layout_for(const ns_ctx* c, int slots_used, bool closure, int schedule, i
   return L;
 }
 
+// The layout of a sweep in an arena of `bytes`.  A store-all sweep keeps its stages where the
+// arena has room for all of them; an arena with the size of the sweep without them (what
+// ns_run_arena_bytes answers after ns_set_pipeline(ctx, 0)) or more runs without.  One that
+// misses the full size by less than a step's entry was meant to be that size and is left too
+// small, so that it is reported and not quietly run slower.
+Layout run_layout(const ns_ctx* c, const ns_run_opts* o, const Planner& P, size_t bytes) {
+  const bool verify = o->verify != 0, pipe = pipelined(c, o->nsteps, o->schedule, o->param, verify);
+  auto layout = [&](int keep_all) {
+    return layout_for(c, P.maxlive, o->mlp != nullptr, o->schedule, o->param, P.maxhost, verify, pipe, keep_all);
+  };
+  if (!keeps_all_stages(c, o->nsteps, o->schedule, verify)) return layout(0);
+  const Layout full = layout(o->nsteps);
+  if (bytes >= full.total || full.total - bytes < 4 * full.stage) return full;
+  return layout(0);
+}
+
 }  // namespace
+
+bool ns_i_arena_fits(const ns_ctx* c, const ns_run_opts* o, size_t bytes) {
+  Planner P;
+  if (make_plan(o->nsteps, o->schedule, o->param, P)) return true;   // refused as a plan, not for its arena
+  return bytes >= run_layout(c, o, P, bytes).total;
+}
 
 extern "C" {
 
@@ -430,10 +452,7 @@ size_t ns_run_arena_bytes(const ns_ctx* c, const ns_run_opts* o) {
   if (!c || !o) return 0;
   Planner P;
   if (make_plan(o->nsteps, o->schedule, o->param, P)) return 0;
-  return layout_for(c, P.maxlive, o->mlp != nullptr, o->schedule, o->param, P.maxhost, o->verify != 0,
-                    pipelined(c, o->nsteps, o->schedule, o->param, o->verify != 0),
-                    keeps_all_stages(c, o->nsteps, o->schedule, o->verify != 0) ? o->nsteps : 0)
-      .total;
+  return run_layout(c, o, P, (size_t)-1).total;
 }
 
 size_t ns_run_host_bytes(const ns_ctx* c, const ns_run_opts* o) {
@@ -899,8 +918,7 @@ static int forward_run_impl(ns_ctx* c, const double* w0, const double* s, const 
     return r;
   }
   S->pipe = pipelined(c, o->nsteps, o->schedule, o->param, o->verify != 0);
-  S->L = layout_for(c, S->P.maxlive, o->mlp != nullptr, o->schedule, o->param, S->P.maxhost, o->verify != 0,
-                    S->pipe, keeps_all_stages(c, o->nsteps, o->schedule, o->verify != 0) ? o->nsteps : 0);
+  S->L = run_layout(c, o, S->P, arena_bytes);
   if (arena_bytes < S->L.total) {
     delete S;
     return NS_ERR_BUDGET;
