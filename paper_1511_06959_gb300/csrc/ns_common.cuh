@@ -182,7 +182,7 @@ struct MarchShape {
   }
   // kernels that march one range per CTA: also sets g.split for march_range (pieces: the
   // kernel takes the split into pieces; otherwise it uses march_even; fixed_cuts: see
-  // k_adj_stage).  The pieces' second
+  // k_adj_stage; most_ctas: the most CTAs of a split in whole waves).  The pieces' second
   // parts are further CTAs that start as slots fall free; they pay while there are few of
   // them (one per column) and the pieces are longer than a range's priming.  128x64x64,
   // adjoint step: 211 us even, 203 us in pieces; with 144 columns on 304 slots (eight
@@ -192,7 +192,7 @@ struct MarchShape {
   // in one range each (456 slots: a second wave with 56 CTAs), 1850 us in this split.
   template <class K>
   cudaError_t get_ranges(K kern, size_t smem, GridDesc& g, const char* env, int& ctas, bool pieces = true,
-                         bool fixed_cuts = false) {
+                         bool fixed_cuts = false, long long most_ctas = 0x7FFFFFFF) {
     long long n = 0;
     const cudaError_t e = slots_of(kern, smem, env, n);
     if (e != cudaSuccess) return e;
@@ -213,7 +213,7 @@ struct MarchShape {
     // planes a slot marches: one wave of all slots, or whole waves of m ranges per column
     long long best = cols <= n ? (g.nz + n / cols - 1) / (n / cols) + MARCH_GAP : 1LL << 62, count = n;
     const int most = g.nz < MARCH_SPLIT ? g.nz : MARCH_SPLIT;
-    for (int m = 1; m <= most; ++m) {
+    for (int m = 1; m <= most && (m == 1 || cols * m <= most_ctas); ++m) {
       const long long cost = ((cols * m + n - 1) / n) * ((g.nz + m - 1) / m + MARCH_GAP);
       if (cost < best) {
         best = cost;

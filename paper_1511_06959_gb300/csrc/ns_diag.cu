@@ -637,10 +637,21 @@ constexpr int NV = 7;   // rho, u1, u2, u3, p, a, b
 static_assert(SP <= 2 * NT, "a plane must fit two load rounds");
 }  // namespace sgk
 
+// Most CTAs of a sigma_1 launch.  Every CTA has a (max, sum) for every box, so the partials
+// grow with the square of the batch: one range per column, or 2048 CTAs (more than are resident,
+// the second parts of pieces included), and the further ranges of a split in whole waves only
+// while all partials together stay within SG_PARTIALS.  (256 boxes of 64x64: 28 MB of them; with
+// room for eight ranges per column everywhere 226 MB.)
+constexpr long long SG_PARTIALS = 1LL << 19;   // pairs of doubles: 8 MB
+long long sigma1_most_ctas(const GridDesc& g, long long cols) {
+  const long long split = cols * (g.nz < MARCH_SPLIT ? g.nz : MARCH_SPLIT), room = SG_PARTIALS / g.batch;
+  const long long more = split < room ? split : room, most = cols > 2048 ? cols : 2048;
+  return more > most ? more : most;
+}
 size_t sigma1_march_ctas_bound(const GridDesc& g) {
   // the padded (bounded) box has one more column on each side
-  const long long cols = (long long)((g.nx + 2 + TX - 1) / TX) * ((g.ny + 2 + sgk::TY - 1) / sgk::TY) * g.batch;
-  return (size_t)(MARCH_SPLIT * cols > 2048 ? MARCH_SPLIT * cols : 2048);
+  return (size_t)sigma1_most_ctas(
+      g, (long long)((g.nx + 2 + TX - 1) / TX) * ((g.ny + 2 + sgk::TY - 1) / sgk::TY) * g.batch);
 }
 
 // TIN: the state's type; a mixed-precision context's FP64 state is rounded as it is loaded
@@ -1263,8 +1274,9 @@ size_t diag_scratch_doubles(const GridDesc& g, int nphi) {
   // two-launch objective: partials, (N/D, sc) per box and 5 doubles per plane face
   const size_t ob = (size_t)2 * RG * g.batch + 2 * (size_t)g.batch + (size_t)g.ny * g.nz * g.batch * 5;
   if (ob > a) a = ob;
-  // sigma_1 statistics: (max, sum) per box for every CTA of the plane-marching launch
-  const size_t sg = 2 * sigma1_march_ctas_bound(g) * (size_t)g.batch;
+  // sigma_1 statistics: (max, sum) per box for every CTA of the plane-marching launch (which
+  // takes no more boxes than a CTA has threads)
+  const size_t sg = g.batch > sgk::NT ? 0 : 2 * sigma1_march_ctas_bound(g) * (size_t)g.batch;
   if (sg > a) a = sg;
   size_t b = (size_t)RG * (nphi > 0 ? nphi : 1);
   return (a > b ? a : b) + 64;
@@ -1335,7 +1347,8 @@ cudaError_t launch_sigma1(const GridDesc& g, const Coef<CT>& c, const TIN* w, fl
   static MarchShape<TX, sgk::TY> shape;
   int ctas = 0;
   GridDesc gm = g;
-  cudaError_t e = shape.get_ranges(k_sigma1<CT, TIN>, smem, gm, nullptr, ctas);
+  cudaError_t e = shape.get_ranges(k_sigma1<CT, TIN>, smem, gm, nullptr, ctas, true, false,
+                                   sigma1_most_ctas(g, shape.columns(g)));
   if (e != cudaSuccess) return e;
   if ((size_t)ctas > sigma1_march_ctas_bound(g)) return cudaErrorInvalidConfiguration;
   if (g.batch > sgk::NT) return cudaErrorInvalidConfiguration;
