@@ -549,8 +549,9 @@ int ns_mlp_infer(ns_ctx* ctx, const void* net, const float* feat, const float* s
 /* One Adam step (lr, beta 0.9 / 0.999, eps 1e-8; step >= 1 counts from 1) on the mean
  * squared error of softplus(MLP(feat[idx[i]])) against target[idx[i]], i < n, with the
  * forward pass quantised exactly as ns_mlp_infer.  loss (device float, may be NULL)
- * receives the minibatch loss before the update.  The first call with n > 4096, or a larger
- * n, allocates the context's training scratch. */
+ * receives the minibatch loss before the update.  Every context holds the training scratch of
+ * 4096 samples (0.7 MB); the first call with a larger n, or a still larger one, allocates a
+ * scratch of its own.  ns_workspace_bytes counts both. */
 int ns_mlp_train_step(ns_ctx* ctx, void* net, const float* feat, const float* target, const int* idx,
                       int n, int step, double lr, float* loss);
 /* Training label: acc[cell] += max(0, v_hat^T M v_hat) / |grad v_hat|^2 with

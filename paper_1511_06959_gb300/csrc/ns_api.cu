@@ -435,7 +435,8 @@ int ns_create(const ns_params* p, void* stream, ns_ctx** out) {
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < ns_ctx::NSTAGE && e == cudaSuccess; ++i) e = cudaMalloc(&c->stage[i], c->field * esz);
   c->scratch_n = std::max(ns::diag_scratch_doubles(c->g, 256), ns::box_means_scratch_doubles(c->g));
-  // behind it the training scratch of an ordinary minibatch (4096 samples, 0.7 MB)
+  // behind it the training scratch of closure.Network's default minibatch (4096 samples,
+  // 0.7 MB), so that its first step allocates nothing
   const size_t train_n = ns::mlp_train_scratch_floats(4096);
   if (e == cudaSuccess) e = cudaMalloc(&c->scratch, c->scratch_n * sizeof(double) + train_n * sizeof(float));
   if (e == cudaSuccess) {
@@ -461,7 +462,8 @@ int ns_create(const ns_params* p, void* stream, ns_ctx** out) {
     ns_destroy(c);
     return NS_ERR_CUDA;
   }
-  c->ws_bytes = ns_ctx::NSTAGE * c->field * esz + c->scratch_n * sizeof(double) + sizeof(unsigned);
+  c->ws_bytes = ns_ctx::NSTAGE * c->field * esz + c->scratch_n * sizeof(double) + train_n * sizeof(float) +
+                sizeof(unsigned);
   c->g.dbg_err = c->err;   // the bounds checks of debug builds report here
   *out = c;
   return NS_OK;
@@ -767,13 +769,17 @@ int ns_mlp_train_step(ns_ctx* c, void* net, const float* feat, const float* targ
   if (!c || !net || !feat || !target || !idx || n < 1 || step < 1 || !(lr > 0)) return NS_ERR_ARG;
   const size_t need = ns::mlp_train_scratch_floats(n);
   if (need > c->train_scratch_n) {
-    if (c->own_train_scratch) cudaFree(c->own_train_scratch);
+    if (c->own_train_scratch) {
+      cudaFree(c->own_train_scratch);
+      c->ws_bytes -= c->train_scratch_n * sizeof(float);
+    }
     c->own_train_scratch = nullptr;
     c->train_scratch = (float*)(c->scratch + c->scratch_n);
     c->train_scratch_n = ns::mlp_train_scratch_floats(4096);
     if (cudaMalloc(&c->own_train_scratch, need * sizeof(float)) != cudaSuccess) return NS_ERR_CUDA;
     c->train_scratch = c->own_train_scratch;
     c->train_scratch_n = need;
+    c->ws_bytes += need * sizeof(float);
   }
   return cuerr(ns::launch_mlp_train_step(net, feat, target, idx, n, step, lr, c->train_scratch, loss, c->st));
 }
