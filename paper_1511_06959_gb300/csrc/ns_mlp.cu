@@ -16,6 +16,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stdint.h>
 
 #include "ns_common.cuh"
 #include "ns_kernels.h"
@@ -306,6 +307,9 @@ __device__ __forceinline__ float2 gelu2(float2 z) {
 constexpr int W1S = 8;    // 32-bit words per row of W1t (16 bf16)
 constexpr int W2S = 36;   // padded row stride of W2t: 64 bf16 = 32 words
 
+// WIDE: the features are read in pairs, which want 8-byte alignment; a caller's array that has
+// only a float's is read one by one.
+template <bool WIDE>
 __global__ void __launch_bounds__(256, 2) k_mlp_infer(long long n, MlpView net, const float* __restrict__ feat,
                                                       const float* __restrict__ sigma1, float scale, float limit_nu,
                                                       float* __restrict__ nu, unsigned* err, bool cap) {
@@ -345,8 +349,12 @@ __global__ void __launch_bounds__(256, 2) k_mlp_infer(long long n, MlpView net, 
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const bool in = r + 8 * i < n;
-      const float2* f = reinterpret_cast<const float2*>(feat + (size_t)(r + 8 * i) * 16);
-      const float2 lo = in ? f[tq] : f2(0.0f, 0.0f), hi = in ? f[tq + 4] : f2(0.0f, 0.0f);
+      const float* f = feat + (size_t)(r + 8 * i) * 16;
+      auto pair = [&](int k) {
+        if constexpr (WIDE) return reinterpret_cast<const float2*>(f)[k];
+        else return f2(f[2 * k], f[2 * k + 1]);
+      };
+      const float2 lo = in ? pair(tq) : f2(0.0f, 0.0f), hi = in ? pair(tq + 4) : f2(0.0f, 0.0f);
       a[i >> 1][i & 1] = pack_bf16(lo.x, lo.y);
       a[i >> 1][2 + (i & 1)] = pack_bf16(hi.x, hi.y);
     }
@@ -820,7 +828,9 @@ cudaError_t launch_mlp_infer(long long n, void* blob, const float* feat, const f
   if (blocks > 2 * 152) blocks = 2 * 152;   // one wave at two resident CTAs per SM
   if (blocks < 1) blocks = 1;
   count_launch();
-  return launch_pdl(k_mlp_infer, dim3((unsigned)blocks), dim3(256), 0, st, n, mlp_view(blob), feat, sigma1, (float)scale, (float)limit_nu, nu, err, cap);
+  const bool wide = ((uintptr_t)feat & 7) == 0;
+  return launch_pdl(wide ? k_mlp_infer<true> : k_mlp_infer<false>, dim3((unsigned)blocks), dim3(256), 0, st, n,
+                    mlp_view(blob), feat, sigma1, (float)scale, (float)limit_nu, nu, err, cap);
 }
 
 // CTAs of a minibatch: whole clusters (the last ones may have no samples)
