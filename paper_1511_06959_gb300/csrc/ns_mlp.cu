@@ -37,38 +37,110 @@ __device__ __forceinline__ float ldf(const double* p, size_t o) { return d2f(p[o
 __device__ __forceinline__ float ldf(const float* p, size_t o) { return p[o]; }
 
 // ------------------------------------------------------------------------------------
-// box means of (rho, u1, u2, u3, p): FP32 per cell, FP64 sums, deterministic
+// box means of (rho, u1, u2, u3, p): FP32 per cell, sums of FP64's precision or better,
+// deterministic
 // ------------------------------------------------------------------------------------
 template <class TIN>
-__global__ void __launch_bounds__(RB) k_box_means(GridDesc g, float gamma, const TIN* __restrict__ w,
+__device__ __forceinline__ void mean_terms(const TIN* __restrict__ w, size_t o, long long cells, float gamma, float x[5]) {
+  const float r = ldf(w, o);
+  const float ir = 1.0f / r;
+  const float u0 = ldf(w, o + cells) * ir, u1 = ldf(w, o + 2 * cells) * ir, u2 = ldf(w, o + 3 * cells) * ir;
+  x[0] = r;
+  x[1] = u0;
+  x[2] = u1;
+  x[3] = u2;
+  x[4] = (gamma - 1.0f) * (ldf(w, o + 4 * cells) - 0.5f * r * (u0 * u0 + u1 * u1 + u2 * u2));
+}
+
+// s = a + b and its rounding error (Knuth's two-sum, exact while nothing overflows)
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+  return s;
+}
+// A float sum with the errors of its additions summed apart, and theirs again (cascaded
+// summation: Rump, Ogita and Oishi's SumK with K = 3): the rounding of lo, below 2^-70 of the
+// terms' magnitude, is all that is lost.
+struct Sum3 {
+  float hi = 0.0f, mid = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float x) {
+    float e, f;
+    hi = two_sum(hi, x, e);
+    mid = two_sum(mid, e, f);
+    lo = __fadd_rn(lo, f);
+  }
+  __device__ __forceinline__ void add(const Sum3& x) {
+    float f;
+    add(x.hi);
+    mid = two_sum(mid, x.mid, f);
+    lo = __fadd_rn(lo, __fadd_rn(x.lo, f));
+  }
+};
+// own += the other half's value, of the two a lane holds: the lanes without the bit o of
+// their number keep a, the others b
+__device__ __forceinline__ Sum3 halve(const Sum3& a, const Sum3& b, int o) {
+  const bool up = (threadIdx.x & o) != 0;
+  Sum3 own = up ? b : a, away = up ? a : b, in;
+  in.hi = __shfl_xor_sync(0xffffffffu, away.hi, o);
+  in.mid = __shfl_xor_sync(0xffffffffu, away.mid, o);
+  in.lo = __shfl_xor_sync(0xffffffffu, away.lo, o);
+  own.add(in);
+  return own;
+}
+
+// The block's sums of the terms in FP64, for values beyond what float sums hold
+template <class TIN>
+__device__ __noinline__ void box_sums_f64(const TIN* __restrict__ w, size_t box, long long cells, float gamma,
+                                          double (*sh)[RB / 32]) {
+  double acc[5] = {0, 0, 0, 0, 0};
+  for (long long i = (long long)blockIdx.x * RB + threadIdx.x; i < cells; i += (long long)gridDim.x * RB) {
+    float x[5];
+    mean_terms(w, box + i, cells, gamma, x);
+    for (int q = 0; q < 5; ++q) acc[q] += (double)x[q];
+  }
+  for (int q = 0; q < 5; ++q) {
+    for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+    if ((threadIdx.x & 31) == 0) sh[q][threadIdx.x >> 5] = acc[q];
+  }
+}
+
+// GB300 issues FP64 additions at 1/64 of the FP32 rate, and a thread has some three cells, so
+// the sums stay in floats (Sum3) until a warp has one value per term: the butterfly across the
+// warp halves the terms a lane keeps (3, 2, 1, then 1 and 1 for lanes of the same term: eight
+// additions in place of 25), and each term's lane makes the FP64 value.  The block falls back
+// to FP64 where a float sum is not finite.  Means and features of 1.77 M cells in eight boxes
+// take 66.5 us, of 256x128x128 cells 183 us, at five CTAs per SM (48 registers: a cell's five
+// loads at once); 70.0 and 217 us at six; 66.3 and 191 us with sums in float pairs, which hold
+// 2^-44 of the terms' magnitude.
+template <class TIN>
+__global__ void __launch_bounds__(RB, 5) k_box_means(GridDesc g, float gamma, const TIN* __restrict__ w,
                                                   double* partial) {
   pdl_enter();
   __shared__ double sh[5][RB / 32];
   const int b = blockIdx.y;
   const size_t box = (size_t)b * 5 * g.cells;
-  // compensated float-pair sums per thread and across the warp (about 2^-44 relative; GB300
-  // issues FP64 additions at 1/64 of the FP32 rate), one FP64 value per warp
-  float hi[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, lo[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+  Sum3 s[5];
   for (long long i = (long long)blockIdx.x * RB + threadIdx.x; i < g.cells; i += (long long)gridDim.x * RB) {
-    const float r = ldf(w, box + i);
-    const float ir = 1.0f / r;
-    const float u0 = ldf(w, box + g.cells + i) * ir, u1 = ldf(w, box + 2 * g.cells + i) * ir,
-                u2 = ldf(w, box + 3 * g.cells + i) * ir;
-    const float p = (gamma - 1.0f) * (ldf(w, box + 4 * g.cells + i) - 0.5f * r * (u0 * u0 + u1 * u1 + u2 * u2));
-    df_add(hi[0], lo[0], r, 0.0f);
-    df_add(hi[1], lo[1], u0, 0.0f);
-    df_add(hi[2], lo[2], u1, 0.0f);
-    df_add(hi[3], lo[3], u2, 0.0f);
-    df_add(hi[4], lo[4], p, 0.0f);
-  }
+    float x[5];
+    mean_terms(w, box + i, g.cells, gamma, x);
 #pragma unroll
-  for (int q = 0; q < 5; ++q) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      df_add(hi[q], lo[q], __shfl_xor_sync(0xffffffffu, hi[q], o), __shfl_xor_sync(0xffffffffu, lo[q], o));
-    if ((threadIdx.x & 31) == 0) sh[q][threadIdx.x >> 5] = f2d(hi[q]) + f2d(lo[q]);
+    for (int q = 0; q < 5; ++q) s[q].add(x[q]);
   }
-  __syncthreads();
+  const Sum3 z;
+  const Sum3 t0 = halve(s[0], s[3], 16), t1 = halve(s[1], s[4], 16), t2 = halve(s[2], z, 16);
+  const Sum3 v0 = halve(t0, t2, 8), v1 = halve(t1, z, 8);
+  Sum3 r = halve(v0, v1, 4);
+  r = halve(r, r, 2);
+  r = halve(r, r, 1);
+  // the term of this lane's sum: the first keeps above had (0, 1, 2) or (3, 4, -), then
+  // (0, 1) or (2, -) of those, then one
+  const int q = ((threadIdx.x & 16) ? 3 : 0) + ((threadIdx.x & 8) ? 2 : 0) + ((threadIdx.x & 4) ? 1 : 0);
+  const bool term = (threadIdx.x & 3) == 0 && (threadIdx.x & 12) != 12 && q < 5;
+  if (term) sh[q][threadIdx.x >> 5] = f2d(r.hi) + (f2d(r.mid) + f2d(r.lo));
+  if (__syncthreads_or(term && !(fabsf(r.hi) < INFINITY && fabsf(r.mid) < INFINITY && fabsf(r.lo) < INFINITY))) {
+    box_sums_f64(w, box, g.cells, gamma, sh);
+    __syncthreads();
+  }
   if (threadIdx.x < 5) {
     double t = 0.0;
 #pragma unroll
@@ -96,7 +168,7 @@ __global__ void __launch_bounds__(RB) k_box_means_final(int nblk, double inv_cel
 // ------------------------------------------------------------------------------------
 // features
 // ------------------------------------------------------------------------------------
-// One CTA takes TX x FY columns and ranges of planes (March) and keeps 1/rho and
+// One CTA takes TX x FY columns and a range of planes (march_range) and keeps 1/rho and
 // rho u of three planes with a one-cell halo in a shared-memory ring, so each cell's state is loaded
 // and divided once per tile instead of seven times; a warp's 32 x 16 features go out
 // through shared memory as whole lines.  1.77 M cells in eight boxes: 115 us with a thread
