@@ -427,17 +427,61 @@ __device__ T sigma1_of(const T M[5][5]) {
 // exactly.  rho and r are taken in FP64 from M; the second term, some 1e-14 of the first, in
 // FP32 with rho for lambda (a third-order change), as r^T (rho - B + v v^T)^-1 r by LDL^T.
 // Its own error is the FP32 roundings (5e-7) over the relative gap g to the next eigenvalue,
-// which 1 / g ~ rel rho / |r|^2 measures: where that would pass 3e-16 (g below about 1e-2),
-// where the squaring has not settled, and for matrices outside FP32's squares, the general
-// iteration takes over.  128x64x64 cells: k_sigma1 in FP64 took 898 us with the general
-// iteration in every cell, 707 us with it started from the FP32 eigenvalue, and 300 us so,
-// with the reciprocals and roots by recip() and root() and the folded entries of M.
+// which 1 / g ~ rel rho / |r|^2 measures: it may reach 3e-16 (g some 1e-2).
+//
+// Where the two largest eigenvalues lie closer (solid rotation has them equal) the squared
+// matrix keeps both: a and b span its two largest directions (pivoted Cholesky), and v is the
+// better of the 2 x 2 problem on them, whose entries' differences are formed in FP64.  The
+// error d of v within the pair, FP32's, counts d^2 g only, and the other direction u is taken
+// out of the second term like v, so that the gap that counts is the one to the third
+// eigenvalue (what couples the two through the rest, another 1e-14, counts only where g is
+// itself that small).  Only where that fails too, and for matrices outside FP32's squares, the general
+// iteration takes over; near a double eigenvalue that one is no better than the root of the
+// rounding (1e-8 of a solid rotation's sigma_1 where the seam or the rounding of M keeps the
+// tridiagonal form from splitting).
+//
+// k_sigma1 in FP64, 128x64x64 cells of random flow, solid rotation, uniform flow: 898, 1324 and
+// 251 us with the general iteration in every cell, 257, 416 and 136 us so, with the
+// reciprocals and roots by recip() and root() and the folded entries of M.
 struct Mat5 {
   double m[5][5];
 };
-__device__ __noinline__ double sigma1_general(Mat5 A) { return sigma1_of<double, 5>(A.m); }
+template <int N>
+__device__ __noinline__ double sigma1_general(Mat5 A) { return sigma1_of<double, N>(A.m); }
 
-__device__ __forceinline__ double sigma1_f64(const double (&M)[5][5]) {
+// column of P (lower triangle) with the largest diagonal entry, over that entry's root
+__device__ __forceinline__ float pivot_column(const float (&P)[5][5], float (&a)[5]) {
+  float pm = P[0][0];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) a[i] = P[i][0];
+#pragma unroll
+  for (int j = 1; j < 5; ++j) {
+    const bool up = P[j][j] > pm;
+    pm = up ? P[j][j] : pm;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) a[i] = up ? (i > j ? P[i][j] : P[j][i]) : a[i];
+  }
+  const float ip = rsqrtf(pm);
+#pragma unroll
+  for (int i = 0; i < 5; ++i) a[i] *= ip;
+  return pm;
+}
+__device__ __forceinline__ void unit5(float (&a)[5]) {
+  float n = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 5; ++i) n = fmaf(a[i], a[i], n);
+  n = rsqrtf(n);
+#pragma unroll
+  for (int i = 0; i < 5; ++i) a[i] *= n;
+}
+__device__ __forceinline__ double dot5(const double (&a)[5], const double (&b)[5]) {
+  double t = a[0] * b[0];
+#pragma unroll
+  for (int i = 1; i < 5; ++i) t = fma(a[i], b[i], t);
+  return t;
+}
+
+__device__ __forceinline__ double sigma1_f64(const double (&M)[5][5], bool flat) {
   float F[5][5], mx = 0.0f;
 #pragma unroll
   for (int i = 0; i < 5; ++i)
@@ -446,117 +490,180 @@ __device__ __forceinline__ double sigma1_f64(const double (&M)[5][5]) {
       F[i][j] = d2f(M[i][j]);
       mx = fmaxf(mx, fabsf(F[i][j]));
     }
-  const float is = 1.0f / mx;
-  float B[5][5], P[5][5], tr = 0.0f;   // lower triangles
+  if (mx == 0.0f) {
+    // no growth at all (uniform flow)
+    unsigned any = 0u;
 #pragma unroll
-  for (int i = 0; i < 5; ++i)
+    for (int i = 0; i < 5; ++i)
 #pragma unroll
-    for (int j = 0; j < 5; ++j) F[i][j] *= is;
-#pragma unroll
-  for (int i = 0; i < 5; ++i)
-#pragma unroll
-    for (int j = 0; j <= i; ++j) {
-      float a = 0.0f;
-#pragma unroll
-      for (int k = 0; k < 5; ++k) a = fmaf(F[k][i], F[k][j], a);
-      B[i][j] = a;
-      if (i == j) tr += a;
-    }
-  const float it = 1.0f / tr;
-#pragma unroll
-  for (int i = 0; i < 5; ++i)
-#pragma unroll
-    for (int j = 0; j <= i; ++j) P[i][j] = B[i][j] * it;
+      for (int j = 0; j < 5; ++j) any |= ((unsigned)__double2hiint(M[i][j]) << 1) | (unsigned)__double2loint(M[i][j]);
+    if (any == 0u) return 0.0;
+  }
   bool ok = false;
-#pragma unroll 1
-  for (int n = 0; n < 10 && !ok; ++n) {
-    float Q[5][5], t = 0.0f;
+  double lam = 0.0;
+  if (mx > 1e-14f && mx < 1e14f) {
+    const float is = 1.0f / mx, is2 = is * is;
+    float B[5][5], P[5][5], tr = 0.0f;   // lower triangles
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+      for (int j = 0; j < 5; ++j) F[i][j] *= is;
 #pragma unroll
     for (int i = 0; i < 5; ++i)
 #pragma unroll
       for (int j = 0; j <= i; ++j) {
-        float a = 0.0f;
+        float t = 0.0f;
 #pragma unroll
-        for (int k = 0; k < 5; ++k) a = fmaf(i > k ? P[i][k] : P[k][i], j > k ? P[j][k] : P[k][j], a);
-        Q[i][j] = a;
-        if (i == j) t += a;
+        for (int k = 0; k < 5; ++k) t = fmaf(F[k][i], F[k][j], t);
+        B[i][j] = t;
+        if (i == j) tr += t;
       }
-    ok = t > 0.9999f;
-    const float q = 1.0f / t;
+    const float it = 1.0f / tr;
+    bool pair = false;
+    int most = 10;
+#pragma unroll 1
+    for (;;) {
 #pragma unroll
-    for (int i = 0; i < 5; ++i)
+      for (int i = 0; i < 5; ++i)
 #pragma unroll
-      for (int j = 0; j <= i; ++j) P[i][j] = Q[i][j] * q;
-  }
-  // v: the column of v v^T with the largest diagonal entry
-  float v[5], vm = P[0][0];
+        for (int j = 0; j <= i; ++j) P[i][j] = B[i][j] * it;
+      bool settled = false;
+      int n = 0;
+#pragma unroll 1
+      for (; n < most && !settled; ++n) {
+        float Q[5][5], t = 0.0f;
 #pragma unroll
-  for (int i = 0; i < 5; ++i) v[i] = P[i][0];
+        for (int i = 0; i < 5; ++i)
 #pragma unroll
-  for (int j = 1; j < 5; ++j) {
-    const bool up = P[j][j] > vm;
-    vm = up ? P[j][j] : vm;
+          for (int j = 0; j <= i; ++j) {
+            float q = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 5; ++i) v[i] = up ? (i > j ? P[i][j] : P[j][i]) : v[i];
-  }
-  const float iv = rsqrtf(vm);
-  double vd[5], vv = 0.0, yy = 0.0, y[5], r[5];
+            for (int k = 0; k < 5; ++k) q = fmaf(i > k ? P[i][k] : P[k][i], j > k ? P[j][k] : P[k][j], q);
+            Q[i][j] = q;
+            if (i == j) t += q;
+          }
+        settled = !pair && t > 0.9999f;
+        const float q = 1.0f / t;
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    v[i] *= iv;
-    vd[i] = f2d(v[i]);
-    vv = fma(vd[i], vd[i], vv);
-  }
+        for (int i = 0; i < 5; ++i)
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    double a = 0.0;
+          for (int j = 0; j <= i; ++j) P[i][j] = Q[i][j] * q;
+      }
+      pair = pair || !settled;
+      float a[5], u[5];
+      const float pa = pivot_column(P, a);
+      double v[5], y[5];
+      if (pair) {
+        // b: the same of what is left of P, orthogonal to a
+        float b[5];
 #pragma unroll
-    for (int j = 0; j < 5; ++j) a = fma(M[i][j], vd[j], a);
-    y[i] = a;
-    yy = fma(a, a, yy);
-  }
-  const double rho = yy * recip(vv);
-  const float is2 = is * is;
-  const float rf = d2f(rho) * is2;
-  float rr = 0.0f, x[5];
+        for (int i = 0; i < 5; ++i)
 #pragma unroll
-  for (int j = 0; j < 5; ++j) {
-    double a = -rho * vd[j];
+          for (int j = 0; j <= i; ++j) P[i][j] = fmaf(-a[i], a[j], P[i][j]);
+        const float pb = pivot_column(P, b);
+        unit5(a);
+        float ab = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 5; ++i) a = fma(M[i][j], y[i], a);
-    r[j] = a;
-    x[j] = d2f(r[j]) * is2;
-    rr = fmaf(x[j], x[j], rr);
-  }
-  // x^T K^-1 x, K = rf I - B + rf v v^T
-  float K[5][5], del = 0.0f;
+        for (int i = 0; i < 5; ++i) ab = fmaf(a[i], b[i], ab);
 #pragma unroll
-  for (int i = 0; i < 5; ++i)
+        for (int i = 0; i < 5; ++i) b[i] = fmaf(-ab, a[i], b[i]);
+        unit5(b);
+        if (!(pb > 1e-5f * pa)) {   // the second direction has been lost: two squarings fewer
+          if (most < 10) break;
+          most = n - 2;
+          continue;
+        }
+        double bd[5], yb[5];
 #pragma unroll
-    for (int j = 0; j <= i; ++j) K[i][j] = fmaf(rf * v[i], v[j], (i == j ? rf : 0.0f) - B[i][j]);
+        for (int i = 0; i < 5; ++i) {
+          v[i] = f2d(a[i]);
+          bd[i] = f2d(b[i]);
+        }
 #pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    ok = ok && K[k][k] > 0.0f;
-    const float id = 1.0f / K[k][k];
-    del = fmaf(x[k] * x[k], id, del);
+        for (int i = 0; i < 5; ++i) {
+          y[i] = dot5(M[i], v);
+          yb[i] = dot5(M[i], bd);
+        }
+        // the pencil (y, yb)^T (y, yb), (v, bd)^T (v, bd) with b less its part q a along a (the
+        // lengths are 1 to 1e-7): half the difference of the diagonal entries and the off-diagonal one
+        const double g11 = dot5(v, v), g12 = dot5(v, bd), q = fma(g12, 1.0 - g11, g12);
+        const double g22 = fma(-q, g12, dot5(bd, bd));
+        const double h11 = dot5(y, y), h12 = dot5(y, yb), h22 = fma(q, fma(q, h11, -2.0 * h12), dot5(yb, yb));
+        const double sc = f2d(is2);
+        const float fd = d2f(0.5 * sc * fma(h11, g22, -h22 * g11)), fo = d2f(sc * fma(-q, h11, h12));
+        const float hyp = sqrtf(fmaf(fd, fd, fo * fo));
+        float c = fd >= 0.0f ? fd + hyp : fo, t = fd >= 0.0f ? fo : hyp - fd;
+        const float n2 = fmaf(c, c, t * t);
+        const float in = n2 > 0.0f ? rsqrtf(n2) : 0.0f;
+        c = n2 > 0.0f ? c * in : 1.0f;   // (equal to rounding: any direction will do)
+        t *= in;
+        const double cb = f2d(t), ca = fma(-cb, q, f2d(c));
 #pragma unroll
-    for (int i = k + 1; i < 5; ++i) {
-      const float l = K[i][k] * id;
-      x[i] = fmaf(-l, x[k], x[i]);
+        for (int i = 0; i < 5; ++i) {
+          v[i] = fma(ca, v[i], cb * bd[i]);
+          y[i] = fma(ca, y[i], cb * yb[i]);
+          u[i] = fmaf(c, b[i], -t * a[i]);
+        }
+      } else {
 #pragma unroll
-      for (int j = k + 1; j <= i; ++j) K[i][j] = fmaf(-l, K[j][k], K[i][j]);
+        for (int i = 0; i < 5; ++i) v[i] = f2d(a[i]);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+          y[i] = dot5(M[i], v);
+          u[i] = 0.0f;
+        }
+      }
+      const double rho = dot5(y, y) * recip(dot5(v, v));
+      const float rf = d2f(rho) * is2;
+      float rr = 0.0f, x[5], vf[5];
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        double r = -rho * v[j];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) r = fma(M[i][j], y[i], r);
+        vf[j] = d2f(v[j]);
+        x[j] = d2f(r) * is2;
+        rr = fmaf(x[j], x[j], rr);
+      }
+      // x^T K^-1 x, K = rf I - B + rf (v v^T + u u^T)
+      float K[5][5], del = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 5; ++i)
+#pragma unroll
+        for (int j = 0; j <= i; ++j)
+          K[i][j] = fmaf(rf * u[i], u[j], fmaf(rf * vf[i], vf[j], (i == j ? rf : 0.0f) - B[i][j]));
+      ok = true;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        ok = ok && K[k][k] > 0.0f;
+        const float id = 1.0f / K[k][k];
+        del = fmaf(x[k] * x[k], id, del);
+#pragma unroll
+        for (int i = k + 1; i < 5; ++i) {
+          const float l = K[i][k] * id;
+          x[i] = fmaf(-l, x[k], x[i]);
+#pragma unroll
+          for (int j = k + 1; j <= i; ++j) K[i][j] = fmaf(-l, K[j][k], K[i][j]);
+        }
+      }
+      lam = fma(rho, f2d(del / rf), rho);
+      ok = ok && del * del <= 6e-10f * rr;
+      if (ok || pair) break;
+      // settled, but the second eigenvalue is too close: again with the pair, two squarings
+      // fewer, after which the second direction has not been lost yet
+      pair = true;
+      most = n - 2;
     }
   }
-  ok = ok && mx > 1e-14f && mx < 1e14f && del * del <= 6e-10f * rr;
   if (!ok) {
     Mat5 A;
 #pragma unroll
     for (int i = 0; i < 5; ++i)
 #pragma unroll
       for (int j = 0; j < 5; ++j) A.m[i][j] = M[i][j];
-    return sigma1_general(A);
+    return flat ? sigma1_general<4>(A) : sigma1_general<5>(A);
   }
-  return root(fma(rho, f2d(del / rf), rho));
+  return root(lam);
 }
 
 // Growth matrix M = M1 - M2 of one cell from central differences of rho, u, p, a, b at
@@ -801,7 +908,7 @@ __global__ void __launch_bounds__(sgk::NT, sizeof(CT) == 4 ? 4 : 1) k_sigma1(Gri
 #pragma unroll
           for (int j = 0; j < 5; ++j) M[3][j] = M[j][3] = CT(0);
         }
-        s1 = sigma1_f64(M);
+        s1 = sigma1_f64(M, g.nz == 1);
       } else {
         CT drho[3], du[3][3], dp[3], da[3], db[3];
 #pragma unroll
