@@ -1174,9 +1174,11 @@ __device__ __forceinline__ T energy_cell(const TIN* __restrict__ w, const TIN* _
 // The same in FP64 with its constants from the host, one reciprocal of r, one square root
 // (m = r c = sqrt(gamma r p)) and one reciprocal of m.  The kernel is bound by its FP64
 // operations: with the constants and the block reduction in every thread of RGS blocks, fewer
-// than two cells each, and quotients, it took 102 us of 128x64x64 cells, against 52 us.
+// than two cells each, and quotients, it took 102 us of 128x64x64 cells, against 49 us.  The
+// constants, each rounded once, are the same in all cells, where the roundings of a cell
+// average out over a box.
 struct EnergyConst {
-  double gamma, gm1, igm1, sg, isg, sgg;   // gamma, gamma - 1, 1 / gm1, sqrt(gamma), 1 / sg, sqrt(gm1 / gamma)
+  double gamma, gm1, sg, k0, k4;   // gamma, gamma - 1, sqrt(gamma), 1 / (gm1 sg), 1 / sqrt(gm1 gamma)
 };
 __device__ __forceinline__ double energy_cell_f64(const double* __restrict__ w, const double* __restrict__ lam,
                                                   size_t box, long long cells, long long i, const EnergyConst& c) {
@@ -1191,9 +1193,9 @@ __device__ __forceinline__ double energy_cell_f64(const double* __restrict__ w, 
   const double m = root(c.gamma * r * p);
   const double y0 = l0 + u0 * l1 + u1 * l2 + u2 * l3 + k * l4;
   const double y1 = l1 + u0 * l4, y2 = l2 + u1 * l4, y3 = l3 + u2 * l4;
-  const double y4 = m * c.igm1 * l4;
-  const double v0 = c.sg * r * r * recip(m) * y0 + c.isg * y4;
-  const double v4 = c.sgg * y4;
+  const double ml = m * l4;
+  const double v0 = c.sg * r * (r * recip(m)) * y0 + c.k0 * ml;
+  const double v4 = c.k4 * ml;
   return v0 * v0 + r * r * (y1 * y1 + y2 * y2 + y3 * y3) + v4 * v4;
 }
 
@@ -1505,8 +1507,8 @@ cudaError_t launch_visc_apply(const GridDesc& g, const double* idx2, const doubl
 }
 
 static EnergyConst energy_const(double gamma) {
-  const double gm1 = gamma - 1.0, sg = sqrt(gamma);
-  return {gamma, gm1, 1.0 / gm1, sg, 1.0 / sg, sqrt(gm1 / gamma)};
+  const long double g = gamma, gm1 = gamma - 1.0, sg = sqrtl(g);
+  return {gamma, gamma - 1.0, (double)sg, (double)(1.0L / (gm1 * sg)), (double)(1.0L / sqrtl(gm1 * g))};
 }
 
 cudaError_t launch_energy(const GridDesc& g, double gamma, double dV, const double* w, const double* lam,
