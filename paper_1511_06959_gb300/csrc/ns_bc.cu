@@ -307,14 +307,25 @@ __device__ __forceinline__ void epilogue_cell(const GridDesc& g, const Pad& P, c
     // FP64 operations bind this kernel, so the weights are formed once per cell and the
     // seed's scale is applied once per component
     const NU* nb = nu + (long long)b * g.cells;
-    const double nc = widen(nb[r]);
     long long q[6] = {r + (x == 0 ? g.nx - 1 : -1), r + (x == g.nx - 1 ? 1 - g.nx : 1),
                       r + (long long)(y == 0 ? g.ny - 1 : -1) * g.nx, r + (long long)(y == g.ny - 1 ? 1 - g.ny : 1) * g.nx,
                       r + (z == 0 ? g.nz - 1 : -1) * g.plane, r + (z == g.nz - 1 ? 1 - g.nz : 1) * g.plane};
     const bool closed[6] = {P.ix && x == 0, P.ix && x == g.nx - 1, P.iy && y == 0, P.iy && y == g.ny - 1, false, false};
+    const NU nc = nb[r];
+    NU nq[6];
+    bool sub = subnormal(nc);   // one test for all seven
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+      nq[d] = nb[q[d]];
+      sub = sub || subnormal(nq[d]);
+    }
     double F[6];
 #pragma unroll
-    for (int d = 0; d < 6; ++d) F[d] = closed[d] ? 0.0 : (nc + widen(nb[q[d]])) * e.hi2[d >> 1];
+    for (int d = 0; d < 6; ++d) F[d] = closed[d] ? 0.0 : (widen(nc) + widen(nq[d])) * e.hi2[d >> 1];
+    if (sub) {
+#pragma unroll
+      for (int d = 0; d < 6; ++d) F[d] = closed[d] ? 0.0 : ((double)nc + (double)nq[d]) * e.hi2[d >> 1];
+    }
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
       const double* Ak = e.A + (long long)b * 5 * g.cells + (long long)k * g.cells;

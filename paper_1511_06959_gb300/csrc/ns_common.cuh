@@ -344,6 +344,17 @@ template <> __device__ __forceinline__ float cvt<float>(double x) { return d2f(x
 template <class T> __device__ __forceinline__ T cvt(float x) { return T(x); }
 __device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ double widen(float x) { return f2d(x); }
+// a caller's float (the added viscosity of FP64 products) exactly, subnormal values too, by
+// the conversion instruction, which issues at FP64's rate
+__device__ __forceinline__ bool subnormal(double) { return false; }   // (doubles are taken as they are)
+__device__ __forceinline__ bool subnormal(float x) {
+  const unsigned a = __float_as_uint(x) << 1;
+  return a - 1u < 0x00FFFFFFu;
+}
+template <class T>
+__device__ __forceinline__ double widen_exact(T x) {
+  return subnormal(x) ? (double)x : widen(x);
+}
 
 // ---------------------------------------------------------------------------------
 // forward-mode dual number (value, tangent) used to build the tangent kernel from

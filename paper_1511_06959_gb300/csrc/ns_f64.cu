@@ -463,7 +463,7 @@ __device__ __forceinline__ void adj_load(AdjPlane& r, const GridDesc& g, size_t 
   if (a.nu) {
 #pragma unroll
     for (int it = 0; it < RND; ++it)
-      if (has_pos(it)) r.n[it] = widen(NS_LD(g, a.nu, nb, h.o[it], n1));
+      if (has_pos(it)) r.n[it] = widen_exact(NS_LD(g, a.nu, nb, h.o[it], n1));
   } else if (a.nud) {
 #pragma unroll
     for (int it = 0; it < RND; ++it)
