@@ -553,11 +553,12 @@ __device__ __forceinline__ void acc_at(int m0, int n0, int q, int& m, int& n) {
   n = n0 + 2 * tq + (q & 1);
 }
 
-// gelu(z) and its derivative from one erf
+// gelu(z) and its derivative from one erf.  The derivative's exponential keeps its subnormal
+// values (|z| above 13.2): they reach the gradients beside a large dL/dy.
 __device__ __forceinline__ void gelu_both(float z, float& h, float& d) {
   const float w = 1.0f + erf_as(z * 0.70710678118654752f);
   h = 0.5f * z * w;
-  d = 0.5f * w + z * exp_ftz(-0.5f * z * z) * 0.39894228040143268f;
+  d = 0.5f * w + z * __expf(-0.5f * z * z) * 0.39894228040143268f;
 }
 
 __global__ void __cluster_dims__(TC, 1, 1) __launch_bounds__(TT) k_mlp_train_partial(MlpView net, const float* __restrict__ feat,
