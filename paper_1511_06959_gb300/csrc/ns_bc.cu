@@ -106,11 +106,23 @@ __device__ __forceinline__ Pad pad_of(const GridDesc& g, const BcDesc& bc) {
   return p;
 }
 
-// Row kernels: one warp per row (a component's y-row of one plane), so that the row's
-// place is worked out once per warp and lanes move along x.  (A thread per element spent
-// most of its time on the 64-bit divisions that split its index: 10.3 us for the field of
-// a 96x48x48 duct.)
-constexpr int BR = 8;   // rows (warps) per CTA
+// Row kernels: a warp takes a row (a component's y-row of one plane), so that the row's place
+// is worked out once and lanes move along x.  (A thread per element spent most of its time on
+// the 64-bit divisions that split its index: 10.3 us for the field of a 96x48x48 duct.)  Of
+// rows up to 16 long it takes as many as its lanes hold.
+constexpr int BR = 8;   // warps per CTA
+__host__ __device__ __forceinline__ int rows_per_warp(int width) { return width > 16 ? 1 : 32 / width; }
+// this lane's place in a warp's rows: which one (rows_per_warp for the lanes left over) and x
+struct RowLane {
+  int row, x;
+};
+__device__ __forceinline__ RowLane row_lane(int width, int rpw) {
+  const int lane = threadIdx.x & 31;
+  RowLane l;
+  l.row = rpw == 1 ? 0 : lane / width;
+  l.x = lane - l.row * width;
+  return l;
+}
 
 // padded fields (interior copied and converted, ghosts zero), ncomp components per box:
 // dst = cvt(scale src); dst2 (may be null) = src unscaled in FP64
@@ -121,14 +133,17 @@ __global__ void __launch_bounds__(32 * BR) k_bc_embed(GridDesc g, BcDesc bc, int
   pdl_enter();
   const Pad P = pad_of(g, bc);
   const long long rows = (long long)P.nyp * g.nz * ncomp * g.batch;
-  const int lane = threadIdx.x & 31;
-  for (long long r = (long long)blockIdx.x * BR + (threadIdx.x >> 5); r < rows; r += (long long)gridDim.x * BR) {
+  const int rpw = rows_per_warp(P.nxp);
+  const RowLane l = row_lane(P.nxp, rpw);
+  if (l.row >= rpw) return;
+  for (long long r = ((long long)blockIdx.x * BR + (threadIdx.x >> 5)) * rpw + l.row; r < rows;
+       r += (long long)gridDim.x * BR * rpw) {
     const long long q = r / P.nyp;                       // (box, component, plane)
     const int y = (int)(r - q * P.nyp) - P.iy;
     const bool in = y >= 0 && y < g.ny;
     const TI* s = src + q * g.plane + (long long)(in ? y : 0) * g.nx;
     TO* d = dst + r * P.nxp;
-    for (int xp = lane; xp < P.nxp; xp += 32) {
+    for (int xp = l.x; xp < P.nxp; xp += 32) {
       const int x = xp - P.ix;
       const double v = in && x >= 0 && x < g.nx ? (double)s[x] : 0.0;
       d[xp] = cvt<TO>(scale * v);
@@ -144,12 +159,15 @@ __global__ void __launch_bounds__(32 * BR) k_bc_crop(GridDesc g, BcDesc bc, int 
   pdl_enter();
   const Pad P = pad_of(g, bc);
   const long long rows = (long long)g.ny * g.nz * ncomp * g.batch;
-  const int lane = threadIdx.x & 31;
-  for (long long r = (long long)blockIdx.x * BR + (threadIdx.x >> 5); r < rows; r += (long long)gridDim.x * BR) {
+  const int rpw = rows_per_warp(g.nx);
+  const RowLane l = row_lane(g.nx, rpw);
+  if (l.row >= rpw) return;
+  for (long long r = ((long long)blockIdx.x * BR + (threadIdx.x >> 5)) * rpw + l.row; r < rows;
+       r += (long long)gridDim.x * BR * rpw) {
     const long long q = r / g.ny;
     const int y = (int)(r - q * g.ny);
     const TI* s = src + q * P.planep + (long long)(y + P.iy) * P.nxp + P.ix;
-    for (int x = lane; x < g.nx; x += 32) dst[r * g.nx + x] = (TO)s[x];
+    for (int x = l.x; x < g.nx; x += 32) dst[r * g.nx + x] = (TO)s[x];
   }
 }
 
@@ -365,14 +383,16 @@ __global__ void __launch_bounds__(32 * BR) k_bc_adj_epilogue(GridDesc g, BcDesc 
                                                              CT* __restrict__ seed, int nbb) {
   pdl_enter();
   const Pad P = pad_of(g, bc);
-  const int lane = threadIdx.x & 31;
   if ((int)blockIdx.x >= nbb) {
-    // 32-cell pieces of rows, one per warp, without the cells next to a boundary
-    const int pieces = (g.nx + 31) / 32;
-    const long long jobs = (long long)pieces * g.ny * g.nz * g.batch, step = (long long)(gridDim.x - nbb) * BR;
-    for (long long j = (long long)(blockIdx.x - nbb) * BR + (threadIdx.x >> 5); j < jobs; j += step) {
+    // 32-cell pieces of rows, one per warp (of rows up to 16 long several), without the cells
+    // next to a boundary
+    const int pieces = (g.nx + 31) / 32, rpw = rows_per_warp(g.nx);
+    const RowLane l = row_lane(g.nx, rpw);
+    if (l.row >= rpw) return;
+    const long long jobs = (long long)pieces * g.ny * g.nz * g.batch, step = (long long)(gridDim.x - nbb) * BR * rpw;
+    for (long long j = ((long long)(blockIdx.x - nbb) * BR + (threadIdx.x >> 5)) * rpw + l.row; j < jobs; j += step) {
       const long long r = j / pieces;
-      const int x = (int)(j - r * pieces) * 32 + lane;
+      const int x = (int)(j - r * pieces) * 32 + l.x;
       const long long q = r / g.ny;
       const int y = (int)(r - q * g.ny);
       const int z = (int)(q % g.nz), b = (int)(q / g.nz);
@@ -461,9 +481,10 @@ long long bc_padded_cells(const GridDesc& g, const BcDesc& bc) {
   return (long long)(g.nx + 2 * bc.inout) * (g.ny + 2 * bc.walls) * g.nz;
 }
 
-// CTAs of the row kernels: BR rows each, at most sixteen per SM (the rest by the stride)
-static unsigned blocks_for_rows(long long rows) {
-  const long long b = (rows + BR - 1) / BR;
+// CTAs of the row kernels: BR warps' rows of this width each, at most sixteen per SM (the rest
+// by the stride)
+static unsigned blocks_for_rows(long long rows, int width) {
+  const long long per = (long long)BR * rows_per_warp(width), b = (rows + per - 1) / per;
   return (unsigned)(b < 152 * 16 ? (b > 0 ? b : 1) : 152 * 16);
 }
 
@@ -472,7 +493,7 @@ cudaError_t launch_bc_embed(const GridDesc& g, const BcDesc& bc, int ncomp, doub
                             cudaStream_t st, double* dst2) {
   const long long rows = (long long)(g.ny + 2 * bc.walls) * g.nz * ncomp * g.batch;
   count_launch();
-  return launch_pdl(k_bc_embed<TO, TI>, dim3(blocks_for_rows(rows)), dim3(32 * BR), 0, st, g, bc, ncomp, scale, src, dst,
+  return launch_pdl(k_bc_embed<TO, TI>, dim3(blocks_for_rows(rows, g.nx + 2 * bc.inout)), dim3(32 * BR), 0, st, g, bc, ncomp, scale, src, dst,
                     dst2);
 }
 
@@ -480,7 +501,7 @@ template <class TO, class TI>
 cudaError_t launch_bc_crop(const GridDesc& g, const BcDesc& bc, int ncomp, const TI* src, TO* dst, cudaStream_t st) {
   const long long rows = (long long)g.ny * g.nz * ncomp * g.batch;
   count_launch();
-  return launch_pdl(k_bc_crop<TO, TI>, dim3(blocks_for_rows(rows)), dim3(32 * BR), 0, st, g, bc, ncomp, src, dst);
+  return launch_pdl(k_bc_crop<TO, TI>, dim3(blocks_for_rows(rows, g.nx)), dim3(32 * BR), 0, st, g, bc, ncomp, src, dst);
 }
 
 template <class T>
@@ -503,7 +524,7 @@ cudaError_t launch_bc_adj_epilogue(const GridDesc& g, const BcDesc& bc, const Bc
   const long long cells = (ncol * g.ny + nrow * (g.nx - ncol)) * g.nz * g.batch;   // next to a boundary
   const long long nbb = (cells + BBT - 1) / BBT;
   if (nbb > (1LL << 30)) return cudaErrorInvalidConfiguration;
-  const unsigned rows = blocks_for_rows((long long)((g.nx + 31) / 32) * g.ny * g.nz * g.batch);
+  const unsigned rows = blocks_for_rows((long long)((g.nx + 31) / 32) * g.ny * g.nz * g.batch, g.nx);
   count_launch();
   return launch_pdl(k_bc_adj_epilogue<CT, NU>, dim3((unsigned)nbb + rows), dim3(32 * BR), 0, st, g, bc, a, W, nu, seed,
                     (int)nbb);
