@@ -508,6 +508,16 @@ template <class T>
 cudaError_t launch_bc_ghosts(const GridDesc& g, const BcDesc& bc, T* W, cudaStream_t st) {
   const long long per = (long long)((bc.inout ? 2 * g.ny : 0) + (bc.walls ? 2 * (g.nx + 2 * bc.inout) : 0)) * g.nz;
   count_launch();
+  // FP64 ghosts are some hundred FP64 instructions a cell, so the CTAs have to spread evenly over
+  // the SMs.  As a dependent launch they are placed while the stage kernel before them, whose two
+  // CTAs fill an SM's registers, is draining: on the SMs that fall free first, four and more
+  // together.  A primal step of 96x48x48 cells with inflow, outflow and walls took 859 us so, of
+  // 20x64x64 cells 666 us; 707 and 413 us launched after it.  (The 2D stage kernels leave room:
+  // 128x128 146 us as a dependent launch, 154 us after it.)
+  if (sizeof(T) == 8 && g.nz > 1) {
+    k_bc_ghosts<T><<<blocks_for(per * g.batch), BB, 0, st>>>(g, bc, W);
+    return cudaGetLastError();
+  }
   return launch_pdl(k_bc_ghosts<T>, dim3(blocks_for(per * g.batch)), dim3(BB), 0, st, g, bc, W);
 }
 
