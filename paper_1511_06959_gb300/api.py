@@ -449,7 +449,8 @@ class Solver:
 
     def set_pipeline(self, on: bool):
         """Pipelined stride sweeps (the next segment replayed on a second stream while the
-        current one is reversed) on or off (ns_set_pipeline); arena_bytes follows."""
+        current one is reversed) and kept stages of store-all sweeps on or off
+        (ns_set_pipeline); arena_bytes follows."""
         _check(self.lib.ns_set_pipeline(self._ctx, int(bool(on))), "ns_set_pipeline")
 
     def last_error(self) -> int:

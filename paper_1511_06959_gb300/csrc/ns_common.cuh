@@ -1,20 +1,23 @@
 // Shared device-side definitions of the NS stencil kernels (sm_103a).
 //
-// Tile geometry: a CTA owns TX x TY cell columns of one box (TX = 32 below; both stage
-// kernels use 32 x 8, their TY set in their own files) and marches a range of
+// Tile geometry: a CTA owns TX x TY cell columns of one box (TX = 32 below; TY is set in each
+// kernel's file: 8 in the stage kernels of ns_rhs.cu and ns_adj.cu, sigma_1 and the features, 4
+// in the FP64 stage kernels of ns_f64.cu) and marches a range of
 // z-planes, keeping a ring of three planes (k-1, k, k+1) of primitive variables with
 // a one-cell halo in x and y in shared memory.  Every face flux of the range is
 // computed once; periodic wrap is resolved when a plane is loaded, so every shared
 // position holds a valid cell even when the box is smaller than the tile.
 //
-// Work split (MarchShape): a launch has as many CTAs as the kernel has resident slots on
-// the device (occupancy calculator x SMs), so that one wave covers the grid, and shares
-// the planes of all tile columns among them.  The FP64 kernels, which have registers to
-// spare, lay the columns end to end, with MARCH_GAP units between two columns for the cost
-// of starting one, and cut that into equal pieces; a CTA marches its piece, range by range
-// where it spans the end of a column (March).  In the FP32 kernels that outer loop costs
-// registers they do not have (the adjoint stage spilled and took 15% longer): there a CTA
-// marches one range (march_range), chosen as get_ranges says.
+// Work split (MarchShape): a launch shares the planes of all tile columns among the kernel's
+// resident slots on the device (occupancy calculator x SMs).  The FP64 stage kernels, which
+// have registers to spare, launch one CTA per slot: they lay the columns end to end, with
+// MARCH_GAP units between two columns for the cost of starting one, and cut that into equal
+// pieces; a CTA marches its piece, range by range where it spans the end of a column (March).
+// In the FP32 kernels that outer loop costs registers they do not have (the adjoint stage
+// spilled and took 15% longer): there a CTA marches one range (march_range), and get_ranges
+// chooses among three launches: the same pieces with the part of each beyond a column's end as
+// a CTA of its own (slots + columns - 1 CTAs), one wave of even ranges (as many CTAs as slots),
+// or several whole waves of equal ranges where the columns outnumber the slots.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -315,9 +318,10 @@ __device__ __forceinline__ double f2d(float f) {
   return __hiloint2double((int)(sign | hi), (int)lo);
 }
 
-// 1/x: the FP32 reciprocal y and y (1 + e + e^2), e = 1 - x y, which cubes its relative error
-// of 2^-22 (three FP64 instructions, the quotient takes some eight); the quotient itself
-// outside FP32's range.
+// 1/x = y / (1 - e), e = 1 - x y, from the FP32 reciprocal y by the geometric series to e^2
+// (Halley's iteration for the reciprocal), which cubes y's relative error of 2^-22: three FP64
+// instructions, the quotient takes some eight, and its value (no difference in 2^24 samples of
+// each of several ranges of exponents); the quotient itself outside FP32's range.
 __device__ __forceinline__ double recip(double x) {
   const float s = d2f(x), a = fabsf(s);
   if (!(a > 1e-30f && a < 1e30f)) return 1.0 / x;
@@ -326,8 +330,8 @@ __device__ __forceinline__ double recip(double x) {
   return fma(y, fma(e, e, e), y);
 }
 
-// sqrt(x) in the same way: t = x y with y = rsqrt(x) of FP32, and t (1 + e/2 + 3 e^2/8),
-// e = 1 - t y
+// sqrt(x) in the same way: t = x y with y = rsqrt(x) of FP32, and t (1 - e)^(-1/2), e = 1 - t y,
+// by the binomial series to 3 e^2/8; within 0.75 units of the last place
 __device__ __forceinline__ double root(double x) {
   const float s = d2f(x);
   if (!(s > 1e-30f && s < 1e30f)) return sqrt(x);

@@ -13,8 +13,9 @@
 //   - divides once per position (the transpose keeps 1/rho).
 // A CTA owns TX x TY columns and marches its piece of planes (March); TY = 4 lets two
 // CTAs of 128 threads share an SM, one computing while the other waits at a barrier.
-// 128x64x64, per stage: residual 386 us before and 224 us now (at the FP64 pipe's full rate
-// for 82% of the time), transpose with the added viscosity 650 us before and 453 us now.
+// 128x64x64, per launch: residual 386 us before and 224 us now (at the FP64 pipe's full rate
+// for 82% of the time), transpose with the added viscosity 650 us before and 422 to 442 us now;
+// a step of four stages 1538 us before and 889 us now, an adjoint step 3720 and 2409 us.
 #include "ns_common.cuh"
 #include "ns_kernels.h"
 
