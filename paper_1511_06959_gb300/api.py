@@ -295,6 +295,7 @@ class Solver:
         self.batch = batch
         self._ctx = ctypes.c_void_p()
         self._graphs = []   # weak references to this context's captured sweeps
+        self._pipeline = os.environ.get("NS_PIPELINE", "1")[:1] != "0"
         st = stream if stream is not None else torch.cuda.current_stream()
         _check(self.lib.ns_create(ctypes.byref(self.params), ctypes.c_void_p(st.cuda_stream),
                                   ctypes.byref(self._ctx)), "ns_create")
@@ -452,6 +453,7 @@ class Solver:
         current one is reversed) and kept stages of store-all sweeps on or off
         (ns_set_pipeline); arena_bytes follows."""
         _check(self.lib.ns_set_pipeline(self._ctx, int(bool(on))), "ns_set_pipeline")
+        self._pipeline = bool(on)
 
     def last_error(self) -> int:
         return int(self.lib.ns_last_error(self._ctx))
@@ -476,6 +478,22 @@ class Solver:
 
     def arena_bytes(self, opts) -> int:
         return int(self.lib.ns_run_arena_bytes(self._ctx, ctypes.byref(opts)))
+
+    def sweep_arena(self, opts, device="cuda"):
+        """The arena of a sweep: arena_bytes(opts) bytes on the device, or, where a store-all
+        sweep's kept stages do not fit there, the bytes without them (the sweep then recomputes
+        them, with the same bits)."""
+        try:
+            return torch.empty(self.arena_bytes(opts), dtype=torch.uint8, device=device)
+        except torch.cuda.OutOfMemoryError:
+            if opts.schedule != NS_CKPT_ALL or not self._pipeline:
+                raise
+        self.set_pipeline(False)
+        try:
+            small = self.arena_bytes(opts)
+        finally:
+            self.set_pipeline(True)
+        return torch.empty(small, dtype=torch.uint8, device=device)
 
     def host_bytes(self, opts) -> int:
         """Host bytes of an NS_CKPT_STRIDE_HOST or NS_CKPT_REVOLVE_HOST sweep's snapshot

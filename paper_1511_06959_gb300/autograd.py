@@ -29,7 +29,7 @@ class SourceProblem:
         if self.phi.shape[1] != solver.cells:
             raise ValueError("phi must hold one value per cell")
         self.opts = solver.run_opts(nsteps, schedule, param, lam_coef, tau)
-        self.arena = torch.empty(solver.arena_bytes(self.opts), dtype=torch.uint8, device=phi.device)
+        self.arena = solver.sweep_arena(self.opts, phi.device)
 
     def source(self, theta: torch.Tensor) -> torch.Tensor:
         """s[b][1] = sum_m theta_m phi_m for every box, zero elsewhere (ns_combine)."""

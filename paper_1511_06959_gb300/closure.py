@@ -145,7 +145,7 @@ def source_sensitivity(S: api.Solver, w0, phi, nsteps, lam_coef=0.0, mlp=None):
     """dJbar/dtheta for the source s = sum theta_m phi_m on x-momentum (theta = 0), and
     the adjoint energy E_vhat(w^0, lam^0), for one closure setting."""
     opts = S.run_opts(nsteps, api.NS_CKPT_ALL, 0, lam_coef, 0.0, True, False, mlp)
-    arena = torch.empty(S.arena_bytes(opts), dtype=torch.uint8, device="cuda")
+    arena = S.sweep_arena(opts)
     J = torch.empty(S.batch, dtype=torch.float64, device="cuda")
     lam0 = torch.empty_like(w0)
     sbar = torch.empty_like(w0)
