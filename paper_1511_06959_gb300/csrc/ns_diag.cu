@@ -430,15 +430,15 @@ __device__ T sigma1_of(const T M[5][5]) {
 // which 1 / g ~ rel rho / |r|^2 measures: it may reach 3e-16 (g some 1e-2).
 //
 // Where the two largest eigenvalues lie closer (solid rotation has them equal) the squared
-// matrix keeps both: a and b span its two largest directions (pivoted Cholesky), and v is the
-// better of the 2 x 2 problem on them, whose entries' differences are formed in FP64.  The
-// error d of v within the pair, FP32's, counts d^2 g only, and the other direction u is taken
-// out of the second term like v, so that the gap that counts is the one to the third
-// eigenvalue (what couples the two through the rest, another 1e-14, counts only where g is
-// itself that small).  Only where that fails too, and for matrices outside FP32's squares, the general
-// iteration takes over; near a double eigenvalue that one is no better than the root of the
-// rounding (1e-8 of a solid rotation's sigma_1 where the seam or the rounding of M keeps the
-// tridiagonal form from splitting).
+// matrix keeps both: a and b span its two largest directions (pivoted Cholesky, whose
+// remainder tells whether there is a third), and v and u are the vectors of the 2 x 2 problem
+// on them, whose entries' differences are formed in FP64.  The same identity for the pair,
+//   lambda = eigenvalue of (rho_v, h; h, rho_u) + (r_v, r_u)^T (lambda - B')^-1 (r_v, r_u),
+// B' off both, has the gap to the third eigenvalue in place of g.  Only where that is too small
+// as well, and for matrices outside FP32's squares, the general iteration takes over; near a
+// multiple eigenvalue that one is no better than the root of the rounding (1e-8 of a solid
+// rotation's sigma_1 where the seam or the rounding of M keeps the tridiagonal form from
+// splitting).
 //
 // k_sigma1 in FP64, 128x64x64 cells of random flow, solid rotation, uniform flow: 898, 1324 and
 // 251 us with the general iteration in every cell, 257, 416 and 136 us so, with the
@@ -550,9 +550,9 @@ __device__ __forceinline__ double sigma1_f64(const double (&M)[5][5], bool flat)
           for (int j = 0; j <= i; ++j) P[i][j] = Q[i][j] * q;
       }
       pair = pair || !settled;
-      float a[5], u[5];
+      float a[5], u[5], z[5], zz = 0.0f, gap = 0.0f, off = 0.0f;
       const float pa = pivot_column(P, a);
-      double v[5], y[5];
+      double v[5], y[5], rho;
       if (pair) {
         // b: the same of what is left of P, orthogonal to a
         float b[5];
@@ -561,6 +561,10 @@ __device__ __forceinline__ double sigma1_f64(const double (&M)[5][5], bool flat)
 #pragma unroll
           for (int j = 0; j <= i; ++j) P[i][j] = fmaf(-a[i], a[j], P[i][j]);
         const float pb = pivot_column(P, b);
+        // the trace of what b leaves in turn
+        float left = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 5; ++i) left += fmaf(-b[i], b[i], P[i][i]);
         unit5(a);
         float ab = 0.0f;
 #pragma unroll
@@ -573,6 +577,7 @@ __device__ __forceinline__ double sigma1_f64(const double (&M)[5][5], bool flat)
           most = n - 2;
           continue;
         }
+        if (!(left < 1e-2f * pb)) break;   // a third one is as large: a and b need not span the largest two
         double bd[5], yb[5];
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
@@ -597,12 +602,29 @@ __device__ __forceinline__ double sigma1_f64(const double (&M)[5][5], bool flat)
         const float in = n2 > 0.0f ? rsqrtf(n2) : 0.0f;
         c = n2 > 0.0f ? c * in : 1.0f;   // (equal to rounding: any direction will do)
         t *= in;
-        const double cb = f2d(t), ca = fma(-cb, q, f2d(c));
+        // v and, in the place of b, u; their quotients' difference, what couples them still, and
+        // u's residual
+        const double vb = f2d(t), va = fma(-vb, q, f2d(c)), ub = f2d(c), ua = fma(-ub, q, -f2d(t));
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
-          v[i] = fma(ca, v[i], cb * bd[i]);
-          y[i] = fma(ca, y[i], cb * yb[i]);
-          u[i] = fmaf(c, b[i], -t * a[i]);
+          const double ai = v[i], yi = y[i];
+          v[i] = fma(va, ai, vb * bd[i]);
+          y[i] = fma(va, yi, vb * yb[i]);
+          bd[i] = fma(ua, ai, ub * bd[i]);
+          yb[i] = fma(ua, yi, ub * yb[i]);
+          u[i] = d2f(bd[i]);
+        }
+        rho = dot5(y, y) * recip(dot5(v, v));
+        const double rhu = dot5(yb, yb) * recip(dot5(bd, bd));
+        gap = d2f(sc * (rho - rhu));
+        off = d2f(sc * fma(-rho, dot5(v, bd), dot5(y, yb)));
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+          double r = -rhu * bd[j];
+#pragma unroll
+          for (int i = 0; i < 5; ++i) r = fma(M[i][j], yb[i], r);
+          z[j] = d2f(r) * is2;
+          zz = fmaf(z[j], z[j], zz);
         }
       } else {
 #pragma unroll
@@ -611,9 +633,10 @@ __device__ __forceinline__ double sigma1_f64(const double (&M)[5][5], bool flat)
         for (int i = 0; i < 5; ++i) {
           y[i] = dot5(M[i], v);
           u[i] = 0.0f;
+          z[i] = 0.0f;
         }
+        rho = dot5(y, y) * recip(dot5(v, v));
       }
-      const double rho = dot5(y, y) * recip(dot5(v, v));
       const float rf = d2f(rho) * is2;
       float rr = 0.0f, x[5], vf[5];
 #pragma unroll
@@ -625,8 +648,8 @@ __device__ __forceinline__ double sigma1_f64(const double (&M)[5][5], bool flat)
         x[j] = d2f(r) * is2;
         rr = fmaf(x[j], x[j], rr);
       }
-      // x^T K^-1 x, K = rf I - B + rf (v v^T + u u^T)
-      float K[5][5], del = 0.0f;
+      // x^T K^-1 x and, for the pair, z^T K^-1 z and x^T K^-1 z, K = rf I - B + rf (v v^T + u u^T)
+      float K[5][5], dv = 0.0f, du = 0.0f, dc = 0.0f;
 #pragma unroll
       for (int i = 0; i < 5; ++i)
 #pragma unroll
@@ -636,18 +659,34 @@ __device__ __forceinline__ double sigma1_f64(const double (&M)[5][5], bool flat)
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         ok = ok && K[k][k] > 0.0f;
-        const float id = 1.0f / K[k][k];
-        del = fmaf(x[k] * x[k], id, del);
+        const float id = 1.0f / K[k][k], xk = x[k] * id, zk = z[k] * id;
+        dv = fmaf(x[k], xk, dv);
+        du = fmaf(z[k], zk, du);
+        dc = fmaf(x[k], zk, dc);
 #pragma unroll
         for (int i = k + 1; i < 5; ++i) {
+          x[i] = fmaf(-K[i][k], xk, x[i]);
+          z[i] = fmaf(-K[i][k], zk, z[i]);
           const float l = K[i][k] * id;
-          x[i] = fmaf(-l, x[k], x[i]);
 #pragma unroll
           for (int j = k + 1; j <= i; ++j) K[i][j] = fmaf(-l, K[j][k], K[i][j]);
         }
       }
-      lam = fma(rho, f2d(del / rf), rho);
-      ok = ok && del * del <= 6e-10f * rr;
+      if (pair) {
+        // the larger eigenvalue of (rho + dv, off + dc; ., rhu + du): ex above the first entry.
+        // w: the most that u can share in its vector, d being du's own error smaller; the
+        // errors of du and dc count by w and its root
+        const float d = gap + (dv - du), o = off + dc, s = sqrtf(fmaf(d, d, 4.0f * o * o));
+        const float ex = d > 0.0f ? 2.0f * o * o / (s + d) : 0.5f * (s - d);
+        const float tv = rr > 0.0f ? dv / rr : 0.0f, tu = zz > 0.0f ? du / zz : 0.0f;
+        const float dl = d - 2e-6f * tu * du;
+        const float w = dl > 0.0f ? fminf(o * o / (dl * dl), 1.0f) : 1.0f;
+        ok = ok && tv * dv + w * tu * du + 2.0f * sqrtf(w) * fabsf(dc) * fmaxf(tv, tu) <= 6e-10f && ex <= 1e-9f * rf;
+        dv += ex;
+      } else {
+        ok = ok && dv * dv <= 6e-10f * rr;
+      }
+      lam = fma(rho, f2d(dv / rf), rho);
       if (ok || pair) break;
       // settled, but the second eigenvalue is too close: again with the pair, two squarings
       // fewer, after which the second direction has not been lost yet
