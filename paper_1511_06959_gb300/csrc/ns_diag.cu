@@ -441,7 +441,7 @@ __device__ T sigma1_of(const T M[5][5]) {
 // splitting).
 //
 // k_sigma1 in FP64, 128x64x64 cells of random flow, solid rotation, uniform flow: 898, 1324 and
-// 251 us with the general iteration in every cell, 257, 416 and 136 us so, with the
+// 251 us with the general iteration in every cell, 266, 510 and 136 us so, with the
 // reciprocals and roots by recip() and root() and the folded entries of M.
 struct Mat5 {
   double m[5][5];
@@ -519,37 +519,38 @@ __device__ __forceinline__ double sigma1_f64(const double (&M)[5][5], bool flat)
         if (i == j) tr += t;
       }
     const float it = 1.0f / tr;
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+      for (int j = 0; j <= i; ++j) P[i][j] = B[i][j] * it;
+    // up to B^1024: v v^T where the second eigenvalue is 2% smaller or more; else the pair at B^512
+    // (one squaring fewer sends the pair's way twice as many cells: random flow in 64x64 cells,
+    // where a warp's slowest lane counts, 33 us and 25 us so)
     bool pair = false;
-    int most = 10;
 #pragma unroll 1
-    for (;;) {
+    for (int n = 0; n <= 9; ++n) {
+      float Q[5][5], t = 0.0f;
 #pragma unroll
       for (int i = 0; i < 5; ++i)
 #pragma unroll
-        for (int j = 0; j <= i; ++j) P[i][j] = B[i][j] * it;
-      bool settled = false;
-      int n = 0;
-#pragma unroll 1
-      for (; n < most && !settled; ++n) {
-        float Q[5][5], t = 0.0f;
+        for (int j = 0; j <= i; ++j) {
+          float q = 0.0f;
 #pragma unroll
-        for (int i = 0; i < 5; ++i)
+          for (int k = 0; k < 5; ++k) q = fmaf(i > k ? P[i][k] : P[k][i], j > k ? P[j][k] : P[k][j], q);
+          Q[i][j] = q;
+          if (i == j) t += q;
+        }
+      const bool settled = t > 0.9999f;
+      pair = n == 9 && !settled;
+      if (pair) break;
+      const float q = 1.0f / t;
 #pragma unroll
-          for (int j = 0; j <= i; ++j) {
-            float q = 0.0f;
+      for (int i = 0; i < 5; ++i)
 #pragma unroll
-            for (int k = 0; k < 5; ++k) q = fmaf(i > k ? P[i][k] : P[k][i], j > k ? P[j][k] : P[k][j], q);
-            Q[i][j] = q;
-            if (i == j) t += q;
-          }
-        settled = !pair && t > 0.9999f;
-        const float q = 1.0f / t;
-#pragma unroll
-        for (int i = 0; i < 5; ++i)
-#pragma unroll
-          for (int j = 0; j <= i; ++j) P[i][j] = Q[i][j] * q;
-      }
-      pair = pair || !settled;
+        for (int j = 0; j <= i; ++j) P[i][j] = Q[i][j] * q;
+      if (settled) break;
+    }
+    do {
       float a[5], u[5], z[5], zz = 0.0f, gap = 0.0f, off = 0.0f;
       const float pa = pivot_column(P, a);
       double v[5], y[5], rho;
@@ -572,12 +573,8 @@ __device__ __forceinline__ double sigma1_f64(const double (&M)[5][5], bool flat)
 #pragma unroll
         for (int i = 0; i < 5; ++i) b[i] = fmaf(-ab, a[i], b[i]);
         unit5(b);
-        if (!(pb > 1e-5f * pa)) {   // the second direction has been lost: two squarings fewer
-          if (most < 10) break;
-          most = n - 2;
-          continue;
-        }
-        if (!(left < 1e-2f * pb)) break;   // a third one is as large: a and b need not span the largest two
+        // a third direction as large: a and b need not span the largest two
+        if (!(pb > 1e-5f * pa && left < 1e-2f * pb)) break;
         double bd[5], yb[5];
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
@@ -687,12 +684,7 @@ __device__ __forceinline__ double sigma1_f64(const double (&M)[5][5], bool flat)
         ok = ok && dv * dv <= 6e-10f * rr;
       }
       lam = fma(rho, f2d(dv / rf), rho);
-      if (ok || pair) break;
-      // settled, but the second eigenvalue is too close: again with the pair, two squarings
-      // fewer, after which the second direction has not been lost yet
-      pair = true;
-      most = n - 2;
-    }
+    } while (false);
   }
   if (!ok) {
     Mat5 A;

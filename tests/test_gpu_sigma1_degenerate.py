@@ -1,6 +1,8 @@
-"""FP64 sigma_1 of flows whose two largest singular values coincide or nearly do: solid
-rotation, in the plane and about an oblique axis, with stretching and with noise from the
-rounding level up, against singular values from numpy."""
+"""FP64 sigma_1 of flows whose largest singular values coincide or nearly do: solid rotation, in
+the plane and about an oblique axis, with noise from the rounding level up, and with an
+expansion that brings a third value near, against singular values from numpy."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -42,3 +44,29 @@ def test_solid_rotation(shape, noise, oblique):
     eps = 2.0 ** -53
     assert np.all(np.abs(host(sig) - ref) <= 100 * eps * 2.0 / min(P.dx) + 20 * eps * ref + 1e-13 * ref)
     assert S.last_error() == 0
+
+
+@pytest.mark.parametrize("delta", [0.0, 1e-6, 1e-5, 1e-4, -1e-4, 1e-3, -1e-3, 3e-3, 1e-2])
+@pytest.mark.parametrize("noise", [1e-9, 3e-7, 1e-5])
+def test_three_singular_values_together(delta, noise):
+    """Rotation with expansion at the rate that puts the double singular value of the rotation
+    within delta of that of the density and pressure rows, and noise about the pair's gap."""
+    api = _api()
+    nx, ny, nz, dx = 64, 48, 40, 0.1
+    z, y, x = np.meshgrid(np.arange(nz), np.arange(ny), np.arange(nx), indexing="ij")
+    r = dx * np.stack([x - nx / 2, y - ny / 2, z - nz / 2])
+    e = 0.05
+    top = np.linalg.norm([[1.5 * e, -1.5 * np.sqrt(0.4) * e], [0.0, 0.9 * e]], 2)
+    om = np.sqrt((top * (1 + delta)) ** 2 - 0.25 * e * e) * np.array([0.6, 0.0, 0.8])
+    u = e * r + np.stack([om[1] * r[2] - om[2] * r[1], om[2] * r[0] - om[0] * r[2], om[0] * r[1] - om[1] * r[0]])
+    u += noise * dx * e * np.random.default_rng(6).standard_normal(u.shape)
+    one = np.ones((nz, ny, nx))
+    w = synth._conservative(one, u, one / 1.4, 1.4)
+    P = dataclasses.replace(params_for(w), dx=(dx,) * 3)
+    S = make_solver(api, w, P, 0)
+    sig = torch.empty(w.shape[1:], dtype=torch.float64, device="cuda")
+    S.growth_sigma1(dev(w), sig)
+    ref = O.sigma1_field(w, P)
+    # the general iteration resolves a triple root of a polynomial to the third root of its
+    # rounding, 4.8e-6 of sigma^2
+    assert np.all(np.abs(host(sig) - ref) <= 2.4e-6 * ref)
